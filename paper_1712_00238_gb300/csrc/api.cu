@@ -38,6 +38,8 @@ struct Prep {  // fixed-shape tables for one grid
     // W times the phase of an unshifted sub-box of half-side s_h (the pruned
     // passes), one per s_h met: (s_h, table)
     std::vector<std::pair<int, void*>> Wsh;
+    // the half-spectrum product table of the searches, per s_h (0: shifted sub-box)
+    std::vector<std::pair<int, void*>> Wh;
 };
 
 struct TimerRec {
@@ -475,10 +477,11 @@ static cudaError_t pass_y_fwd(const Geo& G, const Tw<T>& tw, const cplx<T>* in, 
 }
 
 // last axis (z in 3D, y in 2D): FWD (modes) or FUSED (product with W, inverse)
+// of all modes, or (half) of the half spectrum that a search goes on with
 template <typename T>
 static cudaError_t pass_last(int mode, const Geo& G, const Tw<T>& tw, const cplx<T>* in, int64_t in_rs,
                              cplx<T>* out, int64_t out_rs, const cplx<T>* W, int batch, cudaStream_t st,
-                             int lines = LINES_STD) {
+                             int lines = LINES_STD, bool half = false) {
     ColArgs<T> c{};
     c.lines = lines;
     c.in = in;
@@ -500,21 +503,23 @@ static cudaError_t pass_last(int mode, const Geo& G, const Tw<T>& tw, const cplx
     // by the streaming data: let the batch's rotations share each block of it
     const int64_t w_bytes = (int64_t)c.ncols * G.N * (int64_t)sizeof(cplx<T>);
     c.rot_fastest = ((mode == COL_FUSED || mode == COL_FUSED_P) && w_bytes > ((int64_t)32 << 20)) ? 1 : 0;
+    if (half) return launch_cols_half<T>(mode == COL_FUSED_P, c, batch, st);
     return launch_cols<T>(mode, c, batch, st);
 }
 
-// inverse y (3D): (N,N,N) in place
+// inverse y (3D), in place: (N,N,nx), nx = N, or N/2 of a half spectrum
 template <typename T>
-static cudaError_t pass_y_inv(const Geo& G, const Tw<T>& tw, cplx<T>* buf, int64_t rs, int batch, cudaStream_t st) {
+static cudaError_t pass_y_inv(const Geo& G, const Tw<T>& tw, cplx<T>* buf, int64_t rs, int nx, int batch,
+                              cudaStream_t st) {
     ColArgs<T> c{};
     c.in = buf;
     c.out = buf;
     c.in_rot_stride = rs;
     c.out_rot_stride = rs;
-    c.ncols = G.N;
+    c.ncols = nx;
     c.nouter = G.N;
-    c.in_outer_stride = (int64_t)G.N * G.N;
-    c.out_outer_stride = (int64_t)G.N * G.N;
+    c.in_outer_stride = (int64_t)G.N * nx;
+    c.out_outer_stride = (int64_t)G.N * nx;
     c.len_in = G.N;
     c.s_h = 0;
     c.N = G.N;
@@ -802,9 +807,15 @@ struct Search {
     Plan plan{};
     bool prunable = false;          // pruned forward passes apply (sub-box in the low half of a line)
     bool alt_cols = false;          // and their narrow / wide column plans exist (FP32, n 128..384)
-    const cplx<T>* Wsh = nullptr;   // the shifted table W' of the pruned passes
+    Prep* prep = nullptr;           // the fixed shape's tables on this grid
+    const cplx<T>* Wsh = nullptr;   // the shifted table W' of the pruned passes (full spectrum)
+    const cplx<T>* Wh[2] = {};      // half-spectrum tables: of the shifted sub-box, of the pruned passes
     bool iyx = false;               // inverse y + x in clusters (maps, or one candidate per rotation)
     int k_r = 1;          // candidates per rotation (argmax output)
+    // the inverse runs on half a spectrum (only Re f is kept); the cluster inverse
+    // takes the whole of it and ends with one candidate per rotation
+    bool cluster() const { return iyx && (maps || k_r <= 1); }
+    bool half() const { return !maps && !cluster(); }
     int64_t e0 = 0, e1 = 0, rows_last = 0, Nd = 0;
     cplx<T>* b0 = nullptr;
     cplx<T>* b1 = nullptr;
@@ -859,21 +870,34 @@ static int search_setup(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* movi
     // pruned forward passes: the sub-box must fit in the low half of a line
     S->prunable = ctx->opt_pruned && pruned_len_ok(S->G.n) && S->G.s <= S->G.N;
     S->alt_cols = S->prunable && sizeof(T) == 4 && S->G.n >= 128 && S->G.n <= 384;
-    if (S->prunable) {
-        void* ws = nullptr;
-        for (auto& w : prep->Wsh)
-            if (w.first == S->G.s_h) ws = w.second;
-        if (!ws) {
-            CK(ctx, pool_alloc(&ws, (size_t)S->Nd * sizeof(cplx<T>), st));
-            CK(ctx, launch_wshift<T>((const cplx<T>*)prep->W, S->G.N, S->G.dim, S->G.n, S->G.s_h, (cplx<T>*)ws, st));
-            prep->Wsh.emplace_back(S->G.s_h, ws);
-        }
-        S->Wsh = (const cplx<T>*)ws;
-    }
+    S->prep = prep;
     S->plan.fft = fft_plan_default(ctx, *S);
     S->iyx = ctx->opt_inv_cluster && sizeof(T) == 4 && S->G.dim == 3 && inv_yx_supported(S->G.N);
     if (ctx->opt_spread_box && bins_supported(ctx)) S->plan.bins = SPREAD_BOX;
     if (ctx->opt_spread_fused && spread_x_ok(ctx, *S)) S->plan.bins = SPREAD_X;
+    return SD_OK;
+}
+
+// The product table that a job's plan reads, made on the stream if the fixed shape
+// has not met this grid and sub-box yet.
+template <typename T>
+static int search_tables(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
+    const bool pruned = S->plan.fft != SD_FFT_FULL;
+    const int s_h = pruned ? S->G.s_h : 0;
+    const bool half = S->half();
+    if (!half && !pruned) return SD_OK;  // W itself
+    auto& cache = half ? S->prep->Wh : S->prep->Wsh;
+    void* ws = nullptr;
+    for (auto& w : cache)
+        if (w.first == s_h) ws = w.second;
+    if (!ws) {
+        CK(ctx, pool_alloc(&ws, (size_t)S->Nd * sizeof(cplx<T>), st));
+        if (half) CK(ctx, launch_whalf<T>(S->W, S->G.N, S->G.dim, S->G.n, s_h, (cplx<T>*)ws, st));
+        else CK(ctx, launch_wshift<T>(S->W, S->G.N, S->G.dim, S->G.n, s_h, (cplx<T>*)ws, st));
+        cache.emplace_back(s_h, ws);
+    }
+    if (half) S->Wh[pruned] = (const cplx<T>*)ws;
+    else S->Wsh = (const cplx<T>*)ws;
     return SD_OK;
 }
 
@@ -920,8 +944,7 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
     const Geo& G = S.G;
     const int B = S.plan.B;
     const bool fused_x = S.plan.bins == SPREAD_X;
-    // the cluster inverse ends with one candidate per rotation (or the map)
-    const bool iyx = S.iyx && (S.maps || S.k_r <= 1);
+    const bool iyx = S.cluster(), half = S.half();
     for (int64_t r0 = r_lo; r0 < r_hi; r0 += B) {
         const int b = (int)std::min<int64_t>(B, r_hi - r0);
         if (!fused_x) {
@@ -949,7 +972,7 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
         const int mx = pruned ? ROW_FWD_P : ROW_FWD;
         const int my = pruned ? COL_FWD_P : COL_FWD;
         const int mf = pruned ? COL_FUSED_P : COL_FUSED;
-        const C* Wp = pruned ? S.Wsh : S.W;
+        const C* Wp = half ? S.Wh[pruned] : (pruned ? S.Wsh : S.W);
         if (fused_x) {
             // spreading and the forward x transform in one pass: no sub-box
             PassTimer pt(ctx, SD_PASS_SPREAD_X, s, timed);
@@ -973,17 +996,17 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
             }
             {
                 PassTimer pt(ctx, SD_PASS_FUSED, s, timed);
-                CK(ctx, pass_last<T>(mf, G, S.tw, S.b0, S.e0, S.b1, S.e1, Wp, b, s, lines));
+                CK(ctx, pass_last<T>(mf, G, S.tw, S.b0, S.e0, S.b1, S.e1, Wp, b, s, lines, half));
             }
             if (!iyx) {
                 PassTimer pt(ctx, SD_PASS_INV_Y, s, timed);
-                CK(ctx, pass_y_inv<T>(G, S.tw, S.b1, S.e1, b, s));
+                CK(ctx, pass_y_inv<T>(G, S.tw, S.b1, S.e1, half ? G.N / 2 : G.N, b, s));
             }
             fin = S.b1;
             fin_rs = S.e1;
         } else {
             PassTimer pt(ctx, SD_PASS_FUSED, s, timed);
-            CK(ctx, pass_last<T>(mf, G, S.tw, S.b1, S.e1, S.b0, S.e0, Wp, b, s, lines));
+            CK(ctx, pass_last<T>(mf, G, S.tw, S.b1, S.e1, S.b0, S.e0, Wp, b, s, lines, half));
             fin = S.b0;
             fin_rs = S.e0;
         }
@@ -1009,12 +1032,10 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
             r.part_idx = S.pi;
             // k_r > 1: each block keeps its K >= k_r best (K a power of two, <= 16)
             const int K = S.k_r <= 1 ? 1 : (S.k_r <= 2 ? 2 : (S.k_r <= 4 ? 4 : (S.k_r <= 8 ? 8 : 16)));
-            const int mode = K == 1 ? ROW_INV_ARGMAX
-                                    : (K == 2 ? ROW_INV_TOPK2 : (K == 4 ? ROW_INV_TOPK4 : (K == 8 ? ROW_INV_TOPK8 : ROW_INV_TOPK16)));
             {
                 PassTimer pt(ctx, iyx ? SD_PASS_INV_YX : SD_PASS_INV_X, s, timed);
-                if (iyx) CK(ctx, launch_inv_yx<T>(mode, r, b, &nparts, s));
-                else CK(ctx, launch_rows<T>(mode, r, b, &nparts, s));
+                if (iyx) CK(ctx, launch_inv_yx<T>(ROW_INV_ARGMAX, r, b, &nparts, s));
+                else CK(ctx, launch_rows_half<T>(K, r, b, &nparts, s));
             }
             PassTimer pt(ctx, SD_PASS_REDUCE, s, timed);
             if (K == 1) CK(ctx, launch_reduce_argmax(S.ps, S.pi, nparts, b, r0, S.out, s));
@@ -1077,6 +1098,7 @@ static int autotune(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
     auto trial = [&](const Plan& c) -> int {
         Search<T> t = *S;
         t.plan = c;
+        CKI(search_tables<T>(ctx, &t, st));
         size_t need[8] = {};
         search_need(t, need);
         CKI(ws_reserve(ctx, need));
@@ -1125,6 +1147,7 @@ static int run_search(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* moving
     CKI(search_setup<T>(ctx, fixed, moving, quats, n_r, g, out, maps, st, &S));
     S.k_r = k_r;
     if (ctx->opt_autotune && !ctx->opt_plain && ctx->opt_batch <= 0) CKI(autotune<T>(ctx, &S, st));
+    CKI(search_tables<T>(ctx, &S, st));
     size_t need[8] = {};
     search_need(S, need);
     CKI(ws_reserve(ctx, need));
@@ -1197,6 +1220,7 @@ static int run_pairs(sd_ctx* ctx, const sd_pair_job* jobs, int64_t n_jobs, sd_pa
         const sd_pair_job& J = jobs[j];
         CKI(search_setup<T>(ctx, J.fixed, J.moving, J.quats, J.n_r, &J.grid, J.cand_out, 0, st, &S[j]));
         if (ctx->opt_autotune && !ctx->opt_plain && ctx->opt_batch <= 0) CKI(autotune<T>(ctx, &S[j], st));
+        CKI(search_tables<T>(ctx, &S[j], st));
         char part[256];
         snprintf(part, sizeof part, "|%p,%p,%p,%lld,%d,%.17g,%p,%d,%d,%d", (const void*)J.fixed,
                  (const void*)J.moving, (const void*)J.quats, (long long)J.n_r, J.grid.N, J.grid.L,
@@ -1577,6 +1601,7 @@ int sd_shape_free(sd_shape* s) {
         pool_free(p.W, nullptr);
         pool_free(p.G, nullptr);
         for (auto& w : p.Wsh) pool_free(w.second, nullptr);
+        for (auto& w : p.Wh) pool_free(w.second, nullptr);
     }
     delete s;
     return SD_OK;

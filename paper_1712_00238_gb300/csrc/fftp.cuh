@@ -82,15 +82,22 @@ __device__ __forceinline__ int pidx(int j) {
     else return j;
 }
 
+// A step to run after the first stage's loads are issued (none).
+struct NoHook {
+    __device__ __forceinline__ void operator()() const {}
+};
+
 // Line transforms of NL lines per block of NT threads (see fft_lines_io for the
 // thread layouts).  load(line, i, r) returns first-stage input i + r LEN/R1
 // (called for r < R1/2 only when HALF_IN); emit(line, i, r, v) receives output
 // i + r P of the last stage.  PAD: in-line padding of the shared buffer (needed
 // when a warp's lanes walk one line, LAY_ROW); column layouts use an odd pitch
-// and no padding.  SRC_SMEM: the inputs are already in buf.
+// and no padding.  SRC_SMEM: the inputs are already in buf.  hook() runs once in
+// every thread between the first stage's loads and its butterflies: what it
+// writes to shared memory is visible from the second stage on.
 template <typename C, int LEN, bool INV, int NL, int NT, int LAY, bool PAD, bool SRC_SMEM, bool HALF_IN,
-          int S = 0, int P = 1, typename Load, typename Emit>
-__device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& load, Emit& emit) {
+          int S = 0, int P = 1, typename Load, typename Emit, typename Hook = NoHook>
+__device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& load, Emit& emit, Hook hook = Hook{}) {
     constexpr int R = plan_radix(LEN, S);
     constexpr bool first = (S == 0);
     constexpr bool last = (plan_radix(LEN, S + 1) == 0);
@@ -108,7 +115,15 @@ __device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& lo
             if constexpr (first && !SRC_SMEM) {
 #pragma unroll
                 for (int r = 0; r < (half ? R / 2 : R); ++r) v[q][r] = load(line, i, r);
-            } else {
+            }
+        }
+        if constexpr (first) {
+            if (q == 0) hook();
+        }
+        if (TOT % NT == 0 || t < TOT) {
+            int line, i;
+            butterfly_of<LAY, NL, NB>(t, line, i);
+            if constexpr (!first || SRC_SMEM) {
                 const C* ln = buf + line * ld;
 #pragma unroll
                 for (int r = 0; r < (half ? R / 2 : R); ++r) v[q][r] = ln[pidx<PAD>(i + r * NB)];

@@ -181,6 +181,24 @@ struct ColArgs {
 enum { LINES_STD = 0, LINES_NARROW = 1, LINES_WIDE = 2 };  // standard, half, twice
 template <typename T> cudaError_t launch_cols(int mode, const ColArgs<T>& a, int batch, cudaStream_t st);
 
+// ---- half-spectrum inverse of the search ----------------------------------------
+// A search ranks Re f_N only.  With H = W F2 the product spectrum, Re f_N is the
+// inverse transform of the Hermitian part (H(kappa) + conj H(-kappa)) / 2, of which
+// the modes kappa_x >= 0 suffice: the fused last axis forms it for the N/2 columns
+// kappa_x in [0, N/2) (the Nyquist mode is zero), the inverse y pass runs on
+// those columns, and the inverse x pass packs two real rows into one complex line.
+//   table  two N x (ncols / 2) halves: W(kappa) / 2, then conj W(-kappa) / 2
+//   half   volume (z, ky, kx in [0, N/2)), x fastest
+// launch_cols_half: a.in full columns (ncols of them), a.out and a.W as above;
+// pruned: as COL_FUSED_P (else COL_FUSED).  launch_rows_half: a.nrows rows of N/2
+// modes; keep = 1: each block's (max, lowest index), 2 / 4 / 8 / 16: its best ones.
+template <typename T> cudaError_t launch_cols_half(bool pruned, const ColArgs<T>& a, int batch, cudaStream_t st);
+template <typename T> cudaError_t launch_rows_half(int keep, const RowArgs<T>& a, int batch, int* nparts,
+                                                   cudaStream_t st);
+// The table from W (N^dim), with the phase of an unshifted sub-box (s_h; 0 for none).
+template <typename T>
+cudaError_t launch_whalf(const cplx<T>* W, int N, int dim, int n, int s_h, cplx<T>* out, cudaStream_t st);
+
 // twiddles exp(-2 pi i j / len), computed in FP64
 template <typename T> cudaError_t launch_twiddles(cplx<T>* tw, int len, cudaStream_t st);
 

@@ -1,0 +1,3 @@
+// FP64 instantiation of the half-spectrum inverse passes.
+#include "nufft_half.cuh"
+SD_INSTANTIATE_HALF(double)

@@ -1699,12 +1699,13 @@ __global__ void k_wshift(const cplx<T>* W, int N, int dim, int n, int s_h, cplx<
 // launch helpers
 // ---------------------------------------------------------------------------
 
-// Opt a kernel into more than 48 KiB of dynamic shared memory.  The attribute
+// Opt a kernel into more than 48 KiB of shared memory (dynamic plus the kernel's
+// own static variables, hence the lower line here).  The attribute
 // is one value per kernel and device, so it only ever grows: a launch with less
 // shared memory than the current cap needs no change.
 template <typename K>
 static cudaError_t set_smem(K kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
+    if (bytes <= 32 * 1024) return cudaSuccess;
     static std::mutex mu;
     static std::map<std::pair<int, const void*>, size_t> cap;
     int dev = 0;
