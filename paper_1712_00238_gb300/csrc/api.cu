@@ -507,26 +507,26 @@ static cudaError_t pass_last(int mode, const Geo& G, const Tw<T>& tw, const cplx
     return launch_cols<T>(mode, c, batch, st);
 }
 
-// inverse y (3D), in place: (N,N,nx), nx = N, or N/2 of a half spectrum
+// inverse y (3D): (N,N,N) in place, or (half) from the half volume to packed lines
 template <typename T>
-static cudaError_t pass_y_inv(const Geo& G, const Tw<T>& tw, cplx<T>* buf, int64_t rs, int nx, int batch,
-                              cudaStream_t st) {
+static cudaError_t pass_y_inv(const Geo& G, const Tw<T>& tw, cplx<T>* buf, int64_t rs, int batch, cudaStream_t st,
+                              cplx<T>* packed = nullptr, int64_t packed_rs = 0) {
     ColArgs<T> c{};
     c.in = buf;
-    c.out = buf;
+    c.out = packed ? packed : buf;
     c.in_rot_stride = rs;
-    c.out_rot_stride = rs;
-    c.ncols = nx;
+    c.out_rot_stride = packed ? packed_rs : rs;
+    c.ncols = packed ? G.N / 2 : G.N;
     c.nouter = G.N;
-    c.in_outer_stride = (int64_t)G.N * nx;
-    c.out_outer_stride = (int64_t)G.N * nx;
+    c.in_outer_stride = (int64_t)G.N * c.ncols;
+    c.out_outer_stride = (int64_t)G.N * c.ncols;
     c.len_in = G.N;
     c.s_h = 0;
     c.N = G.N;
     c.n = G.n;
     c.twF = tw.N;
     c.twI = tw.N;
-    return launch_cols<T>(COL_INV, c, batch, st);
+    return packed ? launch_pack_y<T>(c, batch, st) : launch_cols<T>(COL_INV, c, batch, st);
 }
 
 // Bin workspace of one spread batch (slot 6) with bins of tb^d cells: its size
@@ -775,7 +775,7 @@ static int64_t per_rot_elems(const Geo& G, int64_t* e0, int64_t* e1) {
         *e0 = std::max(s * s, N * N);
         *e1 = s * N;
     } else {
-        *e0 = std::max(s * s * s, s * N * N);
+        *e0 = std::max({s * s * s, s * N * N, N * N * N / 2});
         *e1 = std::max(s * s * N, N * N * N);
     }
     return *e0 + *e1;
@@ -1000,10 +1000,10 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
             }
             if (!iyx) {
                 PassTimer pt(ctx, SD_PASS_INV_Y, s, timed);
-                CK(ctx, pass_y_inv<T>(G, S.tw, S.b1, S.e1, half ? G.N / 2 : G.N, b, s));
+                CK(ctx, pass_y_inv<T>(G, S.tw, S.b1, S.e1, b, s, half ? S.b0 : nullptr, S.e0));
             }
-            fin = S.b1;
-            fin_rs = S.e1;
+            fin = half ? S.b0 : S.b1;
+            fin_rs = half ? S.e0 : S.e1;
         } else {
             PassTimer pt(ctx, SD_PASS_FUSED, s, timed);
             CK(ctx, pass_last<T>(mf, G, S.tw, S.b1, S.e1, S.b0, S.e0, Wp, b, s, lines, half));

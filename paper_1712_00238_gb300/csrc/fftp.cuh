@@ -82,9 +82,51 @@ __device__ __forceinline__ int pidx(int j) {
     else return j;
 }
 
-// A step to run after the first stage's loads are issued (none).
+// A row pass's twiddles on their way to shared memory: read into registers before
+// the line loads are issued, stored by the hook after them, so a CTA waits for
+// both at once (column passes read theirs through L1: a warp's lanes walk columns
+// and share each twiddle).
+template <typename C, int NTW, int NT>
+struct TwStage {
+    static constexpr int PER = (NTW + NT - 1) / NT;
+    C r[PER > 0 ? PER : 1];
+    __device__ __forceinline__ void load(const C* g) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int j = threadIdx.x + q * NT;
+            if (NTW % NT == 0 || j < NTW) r[q] = g[j];
+        }
+    }
+    __device__ __forceinline__ void store(C* s) const {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int j = threadIdx.x + q * NT;
+            if (NTW % NT == 0 || j < NTW) s[j] = r[q];
+        }
+    }
+};
+
+// Steps a pass runs inside its transform, once in every thread: loaded() after the
+// first stage's loads are issued (what it writes to shared memory is visible from
+// the second stage on), drained() after the barrier that ends the last stage's
+// reads of the line buffer, before its butterflies.
 struct NoHook {
-    __device__ __forceinline__ void operator()() const {}
+    __device__ __forceinline__ void loaded() const {}
+    __device__ __forceinline__ void drained() const {}
+};
+template <typename F>
+struct LoadedHook : NoHook {
+    F f;
+    __device__ __forceinline__ explicit LoadedHook(F g) : f(g) {}
+    __device__ __forceinline__ void loaded() const { f(); }
+};
+template <typename F, typename G>
+struct Hooks {
+    F f;
+    G g;
+    __device__ __forceinline__ Hooks(F a, G b) : f(a), g(b) {}
+    __device__ __forceinline__ void loaded() const { f(); }
+    __device__ __forceinline__ void drained() const { g(); }
 };
 
 // Line transforms of NL lines per block of NT threads (see fft_lines_io for the
@@ -92,9 +134,7 @@ struct NoHook {
 // (called for r < R1/2 only when HALF_IN); emit(line, i, r, v) receives output
 // i + r P of the last stage.  PAD: in-line padding of the shared buffer (needed
 // when a warp's lanes walk one line, LAY_ROW); column layouts use an odd pitch
-// and no padding.  SRC_SMEM: the inputs are already in buf.  hook() runs once in
-// every thread between the first stage's loads and its butterflies: what it
-// writes to shared memory is visible from the second stage on.
+// and no padding.  SRC_SMEM: the inputs are already in buf.
 template <typename C, int LEN, bool INV, int NL, int NT, int LAY, bool PAD, bool SRC_SMEM, bool HALF_IN,
           int S = 0, int P = 1, typename Load, typename Emit, typename Hook = NoHook>
 __device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& load, Emit& emit, Hook hook = Hook{}) {
@@ -105,6 +145,7 @@ __device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& lo
     constexpr int TOT = NL * NB;
     constexpr int PER = (TOT + NT - 1) / NT;
     constexpr bool half = first && HALF_IN;
+    constexpr int RIN = half ? R / 2 : R;
     C v[PER][R];
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
@@ -112,36 +153,36 @@ __device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& lo
         if (TOT % NT == 0 || t < TOT) {
             int line, i;
             butterfly_of<LAY, NL, NB>(t, line, i);
-            if constexpr (first && !SRC_SMEM) {
+            const C* ln = buf + line * ld;
 #pragma unroll
-                for (int r = 0; r < (half ? R / 2 : R); ++r) v[q][r] = load(line, i, r);
+            for (int r = 0; r < RIN; ++r) {
+                if constexpr (first && !SRC_SMEM) v[q][r] = load(line, i, r);
+                else v[q][r] = ln[pidx<PAD>(i + r * NB)];
             }
         }
-        if constexpr (first) {
-            if (q == 0) hook();
-        }
+    }
+    if constexpr (first) hook.loaded();
+    if constexpr (!first || SRC_SMEM) __syncthreads();  // every read of buf before any write
+    if constexpr (last) hook.drained();
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const int t = threadIdx.x + q * NT;
         if (TOT % NT == 0 || t < TOT) {
             int line, i;
             butterfly_of<LAY, NL, NB>(t, line, i);
-            if constexpr (!first || SRC_SMEM) {
-                const C* ln = buf + line * ld;
+            if constexpr (P > 1) {
+                const C* tws = tw + tw_offset(LEN, S) + (i % P) * (R - 1);
 #pragma unroll
-                for (int r = 0; r < (half ? R / 2 : R); ++r) v[q][r] = ln[pidx<PAD>(i + r * NB)];
-                if constexpr (P > 1) {
-                    const C* tws = tw + tw_offset(LEN, S) + (i % P) * (R - 1);
-#pragma unroll
-                    for (int r = 1; r < R; ++r) {
-                        C w = tws[r - 1];
-                        if (INV) w.y = -w.y;
-                        v[q][r] = cmul(v[q][r], w);
-                    }
+                for (int r = 1; r < R; ++r) {
+                    C w = tws[r - 1];
+                    if (INV) w.y = -w.y;
+                    v[q][r] = cmul(v[q][r], w);
                 }
             }
             if constexpr (half) dft_lowhalf<R, INV>(v[q]);
             else dft<R, INV>(v[q]);
         }
     }
-    if constexpr (!first || SRC_SMEM) __syncthreads();  // every read of buf before any write
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         const int t = threadIdx.x + q * NT;
@@ -162,7 +203,7 @@ __device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& lo
     }
     if constexpr (!last) {
         __syncthreads();
-        fftp_lines<C, LEN, INV, NL, NT, LAY, PAD, SRC_SMEM, HALF_IN, S + 1, P * R>(buf, ld, tw, load, emit);
+        fftp_lines<C, LEN, INV, NL, NT, LAY, PAD, SRC_SMEM, HALF_IN, S + 1, P * R>(buf, ld, tw, load, emit, hook);
     }
 }
 

@@ -119,10 +119,8 @@ cudaError_t launch_spread_x(const SpreadArgs<T>& a, const BinArgs& bn, int nbz, 
 // *_P modes are the pruned forward passes of the search: the sub-box is read
 // unshifted (cell a at position a, a < s <= n/2; the shift is a phase folded
 // into W, see launch_wshift), and only the N = n/2 central modes are computed.
-// ROW_INV_TOPK*: inverse x keeping each block's 2 / 4 / 8 / 16 best translations.
 enum RowMode {
-    ROW_FWD = 0, ROW_INV_ARGMAX = 1, ROW_INV_MAP = 2, ROW_EXPAND = 3, ROW_FWD_P = 4,
-    ROW_INV_TOPK2 = 8, ROW_INV_TOPK4 = 9, ROW_INV_TOPK8 = 10, ROW_INV_TOPK16 = 11
+    ROW_FWD = 0, ROW_INV_ARGMAX = 1, ROW_INV_MAP = 2, ROW_EXPAND = 3, ROW_FWD_P = 4
 };
 enum ColMode { COL_FWD = 0, COL_INV = 1, COL_FUSED = 2, COL_EXPAND = 3, COL_FWD_P = 4, COL_FUSED_P = 5 };
 
@@ -183,15 +181,21 @@ template <typename T> cudaError_t launch_cols(int mode, const ColArgs<T>& a, int
 
 // ---- half-spectrum inverse of the search ----------------------------------------
 // A search ranks Re f_N only.  With H = W F2 the product spectrum, Re f_N is the
-// inverse transform of the Hermitian part (H(kappa) + conj H(-kappa)) / 2, of which
+// inverse transform of the Hermitian part G = (H(kappa) + conj H(-kappa)) / 2, of which
 // the modes kappa_x >= 0 suffice: the fused last axis forms it for the N/2 columns
-// kappa_x in [0, N/2) (the Nyquist mode is zero), the inverse y pass runs on
-// those columns, and the inverse x pass packs two real rows into one complex line.
-//   table  two N x (ncols / 2) halves: W(kappa) / 2, then conj W(-kappa) / 2
-//   half   volume (z, ky, kx in [0, N/2)), x fastest
-// launch_cols_half: a.in full columns (ncols of them), a.out and a.W as above;
-// pruned: as COL_FUSED_P (else COL_FUSED).  launch_rows_half: a.nrows rows of N/2
-// modes; keep = 1: each block's (max, lowest index), 2 / 4 / 8 / 16: its best ones.
+// kappa_x in [0, N/2) (the Nyquist mode is zero) and the inverse y pass runs on those
+// columns.  The last column pass (inverse y in 3D, fused in 2D) packs the rows y and
+// y + N/2 into one complex line X = G_y + i G_(y + N/2) of N modes, whose inverse x
+// transform is f_y + i f_(y + N/2).
+//   table   two N x (ncols / 2) halves: W(kappa) / 2, then conj W(-kappa) / 2
+//   half    volume (z, ky, kx in [0, N/2)), x fastest
+//   packed  lines (z, y in [0, N/2)) of N modes
+// launch_cols_half: a.in full columns (ncols of them), a.W a table, a.out half (3D)
+// or packed (2D: ncols = N); pruned: as COL_FUSED_P (else COL_FUSED).
+// launch_pack_y: inverse y, a.in half to a.out packed (another buffer), nouter = N planes.
+// launch_rows_half: a.nrows rows of the map in packed lines; keep = 1: each block's
+// (max, lowest index), 2 / 4 / 8 / 16: its best ones.
+template <typename T> cudaError_t launch_pack_y(const ColArgs<T>& a, int batch, cudaStream_t st);
 template <typename T> cudaError_t launch_cols_half(bool pruned, const ColArgs<T>& a, int batch, cudaStream_t st);
 template <typename T> cudaError_t launch_rows_half(int keep, const RowArgs<T>& a, int batch, int* nparts,
                                                    cudaStream_t st);

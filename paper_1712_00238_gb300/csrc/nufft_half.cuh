@@ -10,8 +10,10 @@
 //                    G = W/2 FFT(x_c) + conj(W(-kappa))/2 FFT(conj x_c'), and one
 //                    inverse transform serves the two;
 //   inverse y        on N/2 columns (the ordinary pass);
-//   inverse x        two real rows a, b as one complex line X = G_a + i G_b, extended by
-//                    G(-kappa) = conj G(kappa): the line transform returns f_a + i f_b.
+//   inverse y        on N/2 columns; its last stage holds outputs y and y + N/2 of a
+//                    column in one thread and writes them as the modes kappa and -kappa
+//                    of one complex line X = G_y + i G_(y + N/2), X(-kappa) = conj G_y + i conj G_(y + N/2)
+//   inverse x        a plain line transform of X: f_y + i f_(y + N/2)
 // A rotation's inverse work and the bytes it moves after the product are halved,
 // and one inverse z transform in three goes.
 #pragma once
@@ -20,38 +22,77 @@
 
 namespace sd {
 
-// Whether a fused half pass reads its twiddles through L1 instead of shared
-// memory: with them in shared memory a 384-point CTA (line buffer 49 KB, mode
-// buffer 25 KB) would miss a third CTA per SM by 4 KB.  A warp's lanes walk
-// columns, so each twiddle is one broadcast load.
-template <typename T, int LENF>
-__host__ __device__ constexpr bool half_tw_global() { return sizeof(T) == 4 && LENF == 384; }
+// Twiddles in shared memory where that costs no resident CTA: a 384-point CTA (line
+// buffer 49 KB, mode buffer 25 KB) would miss its third, and 512 points (99 KB)
+// measured faster through L1 (12 rotations at N = 256: 1171 against 1273 us; 256 points
+// the other way, 68 rotations at N = 128: 562 against 524).
+template <int LENF>
+__host__ __device__ constexpr bool half_tw_smem() { return LENF <= 256; }
+// The asynchronous copies of the mirror column and the table (see the body) hide two
+// global latencies a CTA: 652 -> 562 us at 256 points, 1354 -> 1171 at 512.  384 points
+// are issue- and register-bound (56 a thread): 1914 us without, 2081 with them.
+template <int LENF>
+__host__ __device__ constexpr bool half_prefetch() { return LENF != 384; }
 
 template <typename T, int LENF, int TC>
 __host__ __device__ constexpr size_t cols_half_smem() {
     return ((size_t)TC * (col_pitch(LENF) + col_pitch(LENF / 2)) +
-            (half_tw_global<T, LENF>() ? 0 : tw_count(LENF) + tw_count(LENF / 2))) * sizeof(cplx<T>);
+            (half_tw_smem<LENF>() ? tw_count(LENF) + tw_count(LENF / 2) : 0)) * sizeof(cplx<T>);
 }
+
+// One complex element from global to shared memory without a register.
+template <typename C>
+__device__ __forceinline__ void copy_async(C* dst, const C* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"((int)sizeof(C)) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// Last-stage emitter of an inverse column transform of LEN points that packs
+// outputs o and o + LEN/2 (radix R even: both in one butterfly) into line o of
+// packed rows: out = packed line 0, kx the column's mode.
+template <typename C, int LEN>
+struct PackEmit {
+    static constexpr int R = plan_last_radix(LEN), PL = LEN / R;
+    static_assert(R % 2 == 0, "a butterfly must hold outputs half a line apart");
+    C* out;
+    int kx;
+    bool ok;
+    C low[R / 2];
+    __device__ __forceinline__ void operator()(int, int i, int r, C v) {
+        using T = decltype(C{}.x);
+        if (r < R / 2) {
+            low[r] = v;
+            return;
+        }
+        if (!ok) return;
+        const C ga = low[r - R / 2];
+        C* line = out + (int64_t)(i + (r - R / 2) * PL) * LEN;
+        if (kx == 0) {  // a real mode, and the Nyquist slot
+            line[0] = mk(ga.x, v.x);
+            line[LEN / 2] = mk(T(0), T(0));
+        } else {
+            line[kx] = mk(ga.x - v.y, ga.y + v.x);
+            line[LEN - kx] = mk(ga.x + v.y, v.x - ga.y);
+        }
+    }
+};
 
 // TC half columns per CTA: forward transform of the columns, then of their
 // conjugated mirrors, products summed in `acc`, inverse transform from there.
-template <typename T, int LENF, int TC, bool PRUNED>
+template <typename T, int LENF, int TC, bool PRUNED, bool PACK>
 __device__ __forceinline__ void cols_half_body(const ColArgs<T>& a) {
     using C = cplx<T>;
     constexpr int LENI = LENF / 2, NH = LENI / 2;
     constexpr int NT = cta_threads_for<LENF>(TC);
     static_assert(NT % TC == 0, "a thread keeps one line through every stage");
     constexpr int LD = col_pitch(LENF), LDA = col_pitch(LENI);
-    constexpr int NTWF = tw_count(LENF), NTWI = tw_count(LENI);
     constexpr int NB1 = LENF / plan_radix(LENF, 0);
-    constexpr int PF = LENF / plan_last_radix(LENF), PI = LENI / plan_last_radix(LENI);
-    constexpr bool TWG = half_tw_global<T, LENF>();
+    constexpr int PFL = LENF / plan_last_radix(LENF), PI = LENI / plan_last_radix(LENI);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     C* acc = buf + TC * LD;
-    C* tws = acc + TC * LDA;
-    const C* twF = TWG ? a.twF : tws;
-    const C* twI = TWG ? a.twI : tws + NTWF;
     const bool rf = a.rot_fastest;
     const int b = rf ? (int)blockIdx.x : (int)blockIdx.z;
     // this thread's line: half column hc = ky NH + kx, its column and its mirror's
@@ -65,7 +106,7 @@ __device__ __forceinline__ void cols_half_body(const ColArgs<T>& a) {
     const C* inB = in + (ky == 0 ? 0 : nky - ky) * LENI + (kx == 0 ? 0 : LENI - kx);
     const C* WA = a.W + hc;
     const C* WB = WA + LENI * hcols;
-    C* out = a.out + (int64_t)b * a.out_rot_stride + hc;
+    C* out = a.out + (int64_t)b * a.out_rot_stride;
     const int s = a.len_in;
     const C zero = mk(T(0), T(0));
     // input position of a line (pruned: cell a at position a; else the shifted sub-box)
@@ -77,80 +118,137 @@ __device__ __forceinline__ void cols_half_body(const ColArgs<T>& a) {
             return e >= LENF ? e - LENF : e;
         }
     };
-    // mode slot of output i + r PF, -1 where it is not kept
+    // mode slot of output i + r PFL, -1 where it is not kept
     auto slot = [&](int i, int r) -> int {
         if constexpr (PRUNED) {
             return kept_out<LENF>(r) ? i + kept_slot<LENF>(r) : -1;
         } else {
-            const int o = i + r * PF;
+            const int o = i + r * PFL;
             return o < LENI / 2 ? o : (o >= LENF - LENI / 2 ? o - LENI : -1);
         }
     };
+    constexpr bool PF = half_prefetch<LENF>();
+    constexpr int R1 = plan_radix(LENF, 0), RL = plan_last_radix(LENF), RIN = PRUNED ? R1 / 2 : R1;
+    const int line = (int)threadIdx.x % TC;
+    const C *twF = a.twF, *twI = a.twI;
+    if constexpr (half_tw_smem<LENF>()) {
+        C* tws = acc + TC * LDA;
+        for (int j = threadIdx.x; j < tw_count(LENF); j += NT) tws[j] = a.twF[j];
+        for (int j = threadIdx.x; j < tw_count(LENI); j += NT) tws[tw_count(LENF) + j] = a.twI[j];
+        twF = tws;
+        twI = tws + tw_count(LENF);
+    }
+    // The mirror column's cells wait in buf (cell e of a line at e TC + line), the
+    // first table half in the mode slots of acc it is multiplied into: both are
+    // copied by the thread that reads them.
     auto loadA = [&](int, int i, int r) -> C {
         const int e = cell(i, r);
         return (ok && e < s) ? inA[e * ncols] : zero;
     };
-    auto emitA = [&](int line, int i, int r, C v) {
+    auto fetchW = [&] {
+#pragma unroll
+        for (int q = 0; q < (TC * PFL + NT - 1) / NT; ++q) {
+            const int t = threadIdx.x + q * NT;
+            if (ok && t < TC * PFL)
+#pragma unroll
+                for (int r = 0; r < RL; ++r) {
+                    const int kp = slot(t / TC, r);
+                    if (kp >= 0) copy_async(acc + line * LDA + kp, WA + kp * hcols);
+                }
+        }
+        copy_commit();
+    };
+    auto fetchB = [&] {
+        copy_wait();  // the table's copies
+#pragma unroll
+        for (int q = 0; q < (TC * NB1 + NT - 1) / NT; ++q) {
+            const int t = threadIdx.x + q * NT;
+            if (ok && t < TC * NB1)
+#pragma unroll
+                for (int r = 0; r < RIN; ++r) {
+                    const int e = cell(t / TC, r);
+                    if (e < s) copy_async(buf + e * TC + line, inB + e * ncols);
+                }
+        }
+        copy_commit();
+    };
+    auto emitA = [&](int, int i, int r, C v) {
         const int kp = slot(i, r);
-        if (kp >= 0 && ok) acc[line * LDA + kp] = cmul(v, WA[kp * hcols]);
+        if (kp >= 0 && ok) {
+            C* g = acc + line * LDA + kp;
+            *g = cmul(v, PF ? *g : WA[kp * hcols]);
+        }
     };
     auto loadB = [&](int, int i, int r) -> C {
         const int e = cell(i, r);
+        if (PF) return (ok && e < s) ? cconj(buf[e * TC + line]) : zero;
         return (ok && e < s) ? cconj(inB[e * ncols]) : zero;
     };
-    auto emitB = [&](int line, int i, int r, C v) {  // the entries this thread wrote in emitA
+    auto emitB = [&](int, int i, int r, C v) {  // the entries this thread wrote in emitA
         const int kp = slot(i, r);
         if (kp >= 0 && ok) {
             C* g = acc + line * LDA + kp;
             *g = cadd(*g, cmul(v, WB[kp * hcols]));
         }
     };
-    auto emit_out = [&](int, int i, int r, C v) {
-        if (ok) out[(i + r * PI) * hcols] = v;
-    };
-    if constexpr (!TWG) {
-        for (int j = threadIdx.x; j < NTWF; j += NT) tws[j] = a.twF[j];
-        for (int j = threadIdx.x; j < NTWI; j += NT) tws[NTWF + j] = a.twI[j];
-        // visible after the barrier between the first two stages
+    if constexpr (PF) {
+        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadA, emitA,
+                                                                          Hooks(fetchW, fetchB));
+        copy_wait();
+        // the barrier of loaded(): every thread has read its cells before buf is rewritten
+        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadB, emitB,
+                                                                          LoadedHook([] { __syncthreads(); }));
+    } else {
+        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadA, emitA);
+        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadB, emitB);
     }
-    fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadA, emitA);
-    // every thread has passed the barrier that follows the last stage's reads of
-    // buf, so the second transform may overwrite it
-    if constexpr (plan_radix(LENF, 1) == 0) __syncthreads();
-    fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadB, emitB);
     __syncthreads();
-    fftp_lines<C, LENI, true, TC, NT, LAY_COL, false, true, false>(acc, LDA, twI, loadA, emit_out);
-}
-
-template <typename T, int LENF, int MB, int TC, bool PRUNED>
-__global__ void __launch_bounds__(cta_threads_for<LENF>(TC), MB) k_cols_half(ColArgs<T> a) {
-    cols_half_body<T, LENF, TC, PRUNED>(a);
-}
-
-// Inverse x of two real rows per line.  src: G_a (LEN/2 modes), then G_b.
-// Input p of the complex line: G_a + i G_b below the Nyquist slot, conj G_a + i conj G_b
-// of mode LEN - p above it; mode 0 is real, the Nyquist slot zero.
-template <typename C, int LEN>
-__device__ __forceinline__ C half_line_input(const C* src, int i, int r) {
-    using T = decltype(C{}.x);
-    constexpr int R1 = plan_radix(LEN, 0), NB1 = LEN / R1, H = LEN / 2;
-    static_assert(R1 % 2 == 0, "first radix must be even");
-    if (r < R1 / 2) {
-        const int p = i + r * NB1;
-        const C ga = src[p], gb = src[H + p];
-        if (r == 0 && i == 0) return mk(ga.x, gb.x);
-        return mk(ga.x - gb.y, ga.y + gb.x);
+    if constexpr (PACK) {
+        PackEmit<C, LENI> emit_out{out, kx, ok};
+        fftp_lines<C, LENI, true, TC, NT, LAY_COL, false, true, false>(acc, LDA, twI, loadA, emit_out);
+    } else {
+        auto emit_out = [&](int, int i, int r, C v) {
+            if (ok) out[(i + r * PI) * hcols + hc] = v;
+        };
+        fftp_lines<C, LENI, true, TC, NT, LAY_COL, false, true, false>(acc, LDA, twI, loadA, emit_out);
     }
-    if (r == R1 / 2 && i == 0) return mk(T(0), T(0));
-    const int q = LEN - (i + r * NB1);
-    const C ga = src[q], gb = src[H + q];
-    return mk(ga.x + gb.y, gb.x - ga.y);
 }
 
-constexpr int HALF_ROW_WAVE = 24;  // CTAs per SM a row pass leaves before its CTAs take more groups
+template <typename T, int LENF, int MB, int TC, bool PRUNED, bool PACK>
+__global__ void __launch_bounds__(cta_threads_for<LENF>(TC), MB) k_cols_half(ColArgs<T> a) {
+    cols_half_body<T, LENF, TC, PRUNED, PACK>(a);
+}
 
-// Row groups of TR lines (2 TR rows) handled by one CTA in turn: its K best are
-// kept in registers across the groups and merged once.
+// Inverse y of half a spectrum (3D): columns (z, kx) of N points from the half
+// volume to packed lines.
+template <typename T, int LEN>
+__global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_inv_min_ctas<T, LEN>()) k_pack_y(ColArgs<T> a) {
+    using C = cplx<T>;
+    constexpr int TC = lines_per_cta<T, LEN>();
+    constexpr int NT = cta_threads<T, LEN>();
+    static_assert(NT % TC == 0, "a thread keeps one line through every stage");
+    constexpr int LD = col_pitch(LEN), NH = LEN / 2;
+    constexpr int NB1 = LEN / plan_radix(LEN, 0);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* buf = reinterpret_cast<C*>(smem_raw);
+    const int kx = blockIdx.x * TC + (int)threadIdx.x % TC;
+    const bool ok = kx < NH;
+    const C* in = a.in + (int64_t)blockIdx.z * a.in_rot_stride + (int64_t)blockIdx.y * (LEN * NH) + kx;
+    const C zero = mk(T(0), T(0));
+    auto load = [&](int, int i, int r) -> C { return ok ? in[(i + r * NB1) * NH] : zero; };
+    PackEmit<C, LEN> emit{a.out + (int64_t)blockIdx.z * a.out_rot_stride + (int64_t)blockIdx.y * (LEN * NH), kx, ok};
+    fftp_lines<C, LEN, true, TC, NT, LAY_COL, false, false, false>(buf, LD, a.twI, load, emit);
+}
+
+// CTAs per SM a row pass leaves before its CTAs take more groups (12 to 48 measure alike).
+constexpr int HALF_ROW_WAVE = 24;
+// Register bound of the row pass: the two rows' running best take it past the 40
+// registers of six CTAs (192 points spilled: 247 us per 20 rotations against 175 at four).
+template <int K>
+__host__ __device__ constexpr int rows_half_min_ctas() { return K == 1 ? 4 : (K <= 4 ? 5 : 0); }
+
+// Inverse x of packed lines.  Row groups of TR lines (2 TR rows) are handled by one
+// CTA in turn: its K best are kept in registers across the groups and merged once.
 template <typename T, int LEN, int K>
 __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
     using C = cplx<T>;
@@ -158,12 +256,15 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
     constexpr int NT = cta_threads<T, LEN>();
     constexpr int LD = line_pitch(LEN);
     constexpr int NTW = tw_count(LEN);
+    constexpr int NB1 = LEN / plan_radix(LEN, 0);
     constexpr int PL = LEN / plan_last_radix(LEN);
     constexpr bool one_bfly = TR * (LEN / plan_last_radix(LEN)) <= NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     C* tw = buf + TR * LD;
-    for (int j = threadIdx.x; j < NTW; j += NT) tw[j] = a.tw[j];  // visible from the second stage on
+    TwStage<C, NTW, NT> tws;
+    tws.load(a.tw);
+    constexpr int NH = LEN / 2;
     const C* in = a.in + (int64_t)blockIdx.y * a.in_rot_stride;
     const int nlines = a.nrows / 2, ngroups = (nlines + TR - 1) / TR;
     const C zero = mk(T(0), T(0));
@@ -176,25 +277,28 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
         const int nl = nlines - line0;
         const C* src = in + (int64_t)line0 * LEN;
         auto load = [&](int line, int i, int r) -> C {
-            return line < nl ? half_line_input<C, LEN>(src + line * LEN, i, r) : zero;
+            return line < nl ? src[line * LEN + i + r * NB1] : zero;
         };
         auto emit = [&](int line, int i, int r, C v) {
             if (line >= nl) return;
-            const int o = 2 * (line0 + line) * LEN + i + r * PL;
+            // line (z, y), y < N/2, holds rows (z, y) and (z, y + N/2)
+            const int l = line0 + line, o = (l + l / NH * NH) * LEN + i + r * PL;
             if constexpr (K > 1) {
                 top.push(v.x, o);
-                top.push(v.y, o + LEN);
+                top.push(v.y, o + NH * LEN);
             } else if constexpr (one_bfly) {
                 // outputs (and groups) come in increasing index order: a strict
                 // comparison keeps the lowest index of equal values
                 if (v.x > bestA) { bestA = v.x; idxA = o; }
-                if (v.y > bestB) { bestB = v.y; idxB = o + LEN; }
+                if (v.y > bestB) { bestB = v.y; idxB = o + NH * LEN; }
             } else {
                 argmax_merge(bestA, idxA, v.x, o);
-                argmax_merge(bestB, idxB, v.y, o + LEN);
+                argmax_merge(bestB, idxB, v.y, o + NH * LEN);
             }
         };
-        fftp_lines<C, LEN, true, TR, NT, LAY_ROW, true, false, false>(buf, LD, tw, load, emit);
+        fftp_lines<C, LEN, true, TR, NT, LAY_ROW, true, false, false>(buf, LD, tw, load, emit, LoadedHook([&] {
+            if (g == (int)blockIdx.x) tws.store(tw);
+        }));
         // the next group's first writes to buf come after the barrier that follows
         // this group's last reads
     }
@@ -221,7 +325,7 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
 }
 
 template <typename T, int LEN, int K>
-__global__ void __launch_bounds__(cta_threads<T, LEN>(), K == 1 ? rows_inv_min_ctas<T, LEN>() : 0)
+__global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_half_min_ctas<K>())
 k_rows_half(RowArgs<T> a) {
     rows_half_body<T, LEN, K>(a);
 }
@@ -256,13 +360,13 @@ __global__ void k_whalf(const cplx<T>* W, int N, int dim, int n, int s_h, cplx<T
 
 // ---------------------------------------------------------------------------
 
-template <typename T, int LENF, int TC, int MB, bool PRUNED>
+template <typename T, int LENF, int TC, int MB, bool PRUNED, bool PACK = false>
 static cudaError_t cols_half_launch(const ColArgs<T>& a, int batch, cudaStream_t st) {
     const int hcols = a.ncols / 2;
     const int nb = (hcols + TC - 1) / TC;
     if (nb == 0 || batch == 0) return cudaSuccess;
-    if (a.nouter != 1 || a.N != LENF / 2 || a.ncols % a.N != 0) return cudaErrorInvalidValue;
-    auto kern = k_cols_half<T, LENF, MB, TC, PRUNED>;
+    if (a.nouter != 1 || a.N != LENF / 2 || a.ncols != (PACK ? a.N : a.N * a.N)) return cudaErrorInvalidValue;
+    auto kern = k_cols_half<T, LENF, MB, TC, PRUNED, PACK>;
     constexpr size_t smem = cols_half_smem<T, LENF, TC>();
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
@@ -276,6 +380,8 @@ static cudaError_t cols_half_launch(const ColArgs<T>& a, int batch, cudaStream_t
 template <typename T, int LENF>
 static cudaError_t cols_half_pruned(const ColArgs<T>& a, int batch, cudaStream_t st) {
     static_assert(prunable_len(LENF), "length not prunable");
+    if (a.ncols == a.N)  // 2D: N/2 columns in all, one width
+        return cols_half_launch<T, LENF, lines_per_cta<T, LENF>(), pruned_min_ctas<T, LENF, 2>(), true, true>(a, batch, st);
     if constexpr (alt_cols_ok<T, LENF>()) {
         if (a.lines == LINES_NARROW)
             return cols_half_launch<T, LENF, alt_lines<T, LENF, 0>(), alt_min_ctas<T, LENF, 2, 0>(), true>(a, batch, st);
@@ -298,11 +404,40 @@ cudaError_t launch_cols_half_t(bool pruned, const ColArgs<T>& a, int batch, cuda
         return cudaErrorInvalidValue;
     }
     switch (a.n) {
-#define SD_HALFF_CASE(L) \
-    case L: return cols_half_launch<T, L, lines_per_cta<T, L>(), min_ctas_per_sm<T, L>(), false>(a, batch, st);
+#define SD_HALFF_CASE(L)                                                                                          \
+    case L:                                                                                                       \
+        return a.ncols == a.N                                                                                     \
+                   ? cols_half_launch<T, L, lines_per_cta<T, L>(), min_ctas_per_sm<T, L>(), false, true>(a, batch, st) \
+                   : cols_half_launch<T, L, lines_per_cta<T, L>(), min_ctas_per_sm<T, L>(), false>(a, batch, st);
         SD_HALFF_CASE(16) SD_HALFF_CASE(32) SD_HALFF_CASE(48) SD_HALFF_CASE(64) SD_HALFF_CASE(96)
         SD_HALFF_CASE(128) SD_HALFF_CASE(192) SD_HALFF_CASE(256) SD_HALFF_CASE(384) SD_HALFF_CASE(512)
 #undef SD_HALFF_CASE
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <typename T, int LEN>
+static cudaError_t pack_y_launch(const ColArgs<T>& a, int batch, cudaStream_t st) {
+    constexpr int TC = lines_per_cta<T, LEN>();
+    if (batch == 0) return cudaSuccess;
+    if (a.nouter != LEN || a.ncols != LEN / 2 || a.in == a.out) return cudaErrorInvalidValue;
+    const size_t smem = (size_t)TC * col_pitch(LEN) * sizeof(cplx<T>);
+    auto kern = k_pack_y<T, LEN>;
+    cudaError_t e = set_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3((LEN / 2 + TC - 1) / TC, LEN, batch), cta_threads<T, LEN>(), smem, st>>>(a);
+    note_launch();
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_pack_y_t(const ColArgs<T>& a, int batch, cudaStream_t st) {
+    switch (a.N) {
+#define SD_PACK_CASE(L) \
+    case L: return pack_y_launch<T, L>(a, batch, st);
+        SD_PACK_CASE(8) SD_PACK_CASE(16) SD_PACK_CASE(24) SD_PACK_CASE(32) SD_PACK_CASE(48) SD_PACK_CASE(64)
+        SD_PACK_CASE(96) SD_PACK_CASE(128) SD_PACK_CASE(192) SD_PACK_CASE(256)
+#undef SD_PACK_CASE
     }
     return cudaErrorInvalidValue;
 }
@@ -366,6 +501,9 @@ cudaError_t launch_whalf_t(const cplx<T>* W, int N, int dim, int n, int s_h, cpl
     namespace sd {                                                                                             \
     template <> cudaError_t launch_cols_half<T>(bool pruned, const ColArgs<T>& a, int batch, cudaStream_t st) { \
         return launch_cols_half_t<T>(pruned, a, batch, st);                                                    \
+    }                                                                                                          \
+    template <> cudaError_t launch_pack_y<T>(const ColArgs<T>& a, int batch, cudaStream_t st) {                \
+        return launch_pack_y_t<T>(a, batch, st);                                                               \
     }                                                                                                          \
     template <> cudaError_t launch_rows_half<T>(int keep, const RowArgs<T>& a, int batch, int* np, cudaStream_t st) { \
         return launch_rows_half_t<T>(keep, a, batch, np, st);                                                  \

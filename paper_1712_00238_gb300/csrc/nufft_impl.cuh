@@ -1121,7 +1121,7 @@ __device__ __forceinline__ void block_argmax(T& best, int& bidx) {
     }
 }
 
-// Row passes: TR consecutive rows of one rotation per CTA.
+// Row passes (forward, expand): TR consecutive rows of one rotation per CTA.
 template <typename T, int LEN, int MODE>
 __device__ __forceinline__ void rows_body(const RowArgs<T>& a) {
     using C = cplx<T>;
@@ -1148,36 +1148,22 @@ __device__ __forceinline__ void rows_body(const RowArgs<T>& a) {
             int e = pos + a.s_h;
             if (e >= LEN) e -= LEN;
             return e < a.len_in ? src[e] : zero;
-        } else if constexpr (MODE == ROW_EXPAND) {
+        } else {
             const int e = pos < hN ? pos : (pos >= LEN - hN ? pos - LEN + N : -1);
             return e >= 0 ? src[e] : zero;
-        } else {
-            return src[pos];
         }
     };
-    T best = -INFINITY;
-    int bidx = INT_MAX;
     auto emit = [&](int line, int o, C v) {
         const int row = row0 + line;
         if (row >= a.nrows) return;
         if constexpr (MODE == ROW_FWD) {
             const int kp = o < hN ? o : (o >= LEN - hN ? o - LEN + N : -1);
             if (kp >= 0) out[(int64_t)row * a.out_row_stride + kp] = v;
-        } else if constexpr (MODE == ROW_INV_ARGMAX) {
-            argmax_merge(best, bidx, v.x, row * LEN + o);
         } else {
             out[(int64_t)row * a.out_row_stride + o] = v;
         }
     };
     fft_lines_io<C, LEN, INV, TR, cta_threads<T, LEN>(), LAY_ROW, false>(buf, LD, tw, load, emit);
-    if constexpr (MODE == ROW_INV_ARGMAX) {
-        block_argmax(best, bidx);
-        if (threadIdx.x == 0) {
-            const int64_t o = (int64_t)b * gridDim.x + blockIdx.x;
-            a.part_score[o] = (double)best;
-            a.part_idx[o] = bidx;
-        }
-    }
 }
 
 template <typename T, int LEN, int MODE>
@@ -1302,8 +1288,8 @@ __device__ __forceinline__ void rows_fwd_p_body(const RowArgs<T>& a) {
     C* buf = reinterpret_cast<C*>(smem_raw);
     C* tw = buf + TR * LD;
     const int row0 = blockIdx.x * TR;
-    for (int j = threadIdx.x; j < NTW; j += blockDim.x) tw[j] = a.tw[j];
-    __syncthreads();
+    TwStage<C, NTW, cta_threads<T, LEN>()> tws;
+    tws.load(a.tw);
     const int rs = a.in_row_stride;
     const C* in = a.in + (int64_t)blockIdx.y * a.in_rot_stride + (int64_t)row0 * rs;
     C* out = a.out + (int64_t)blockIdx.y * a.out_rot_stride + (int64_t)row0 * NH;
@@ -1317,7 +1303,8 @@ __device__ __forceinline__ void rows_fwd_p_body(const RowArgs<T>& a) {
     auto emit = [&](int line, int i, int r, C v) {
         if (kept_out<LEN>(r) && line < nrows) out[line * NH + i + kept_slot<LEN>(r)] = v;
     };
-    fftp_lines<C, LEN, false, TR, cta_threads<T, LEN>(), LAY_ROW, true, false, true>(buf, LD, tw, load, emit);
+    fftp_lines<C, LEN, false, TR, cta_threads<T, LEN>(), LAY_ROW, true, false, true>(buf, LD, tw, load, emit,
+                                                                                     LoadedHook([&] { tws.store(tw); }));
 }
 
 template <typename T, int LEN, int MB>
@@ -1332,14 +1319,10 @@ __device__ __forceinline__ void cols_fwd_p_body(const ColArgs<T>& a) {
     using C = cplx<T>;
     constexpr int NT = cta_threads_for<LEN>(TC);
     constexpr int LD = col_pitch(LEN);
-    constexpr int NTW = tw_count(LEN);
     constexpr int NB1 = LEN / plan_radix(LEN, 0);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
-    C* tw = buf + TC * LD;
     const int col0 = blockIdx.x * TC;
-    for (int j = threadIdx.x; j < NTW; j += blockDim.x) tw[j] = a.twF[j];
-    __syncthreads();
     const int ncols = a.ncols;
     const int ncl = ncols - col0;
     const C* in = a.in + (int64_t)blockIdx.z * a.in_rot_stride + (int64_t)blockIdx.y * a.in_outer_stride + col0;
@@ -1353,7 +1336,7 @@ __device__ __forceinline__ void cols_fwd_p_body(const ColArgs<T>& a) {
     auto emit = [&](int line, int i, int r, C v) {
         if (kept_out<LEN>(r) && line < ncl) out[(i + kept_slot<LEN>(r)) * ncols + line] = v;
     };
-    fftp_lines<C, LEN, false, TC, NT, LAY_COL, false, false, true>(buf, LD, tw, load, emit);
+    fftp_lines<C, LEN, false, TC, NT, LAY_COL, false, false, true>(buf, LD, a.twF, load, emit);
 }
 
 template <typename T, int LEN, int MB, int TC>
@@ -1429,15 +1412,11 @@ __device__ __forceinline__ void cols_inv_p_body(const ColArgs<T>& a) {
     constexpr int TC = lines_per_cta<T, LEN>();
     constexpr int NT = cta_threads<T, LEN>();
     constexpr int LD = col_pitch(LEN);
-    constexpr int NTW = tw_count(LEN);
     constexpr int NB1 = LEN / plan_radix(LEN, 0);
     constexpr int PL = LEN / plan_last_radix(LEN);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
-    C* tw = buf + TC * LD;
     const int col0 = blockIdx.x * TC;
-    for (int j = threadIdx.x; j < NTW; j += blockDim.x) tw[j] = a.twF[j];
-    __syncthreads();
     const int ncols = a.ncols;
     const int ncl = ncols - col0;
     const C* in = a.in + (int64_t)blockIdx.z * a.in_rot_stride + (int64_t)blockIdx.y * a.in_outer_stride + col0;
@@ -1447,7 +1426,7 @@ __device__ __forceinline__ void cols_inv_p_body(const ColArgs<T>& a) {
     auto emit = [&](int line, int i, int r, C v) {
         if (line < ncl) out[(i + r * PL) * ncols + line] = v;
     };
-    fftp_lines<C, LEN, true, TC, NT, LAY_COL, false, false, false>(buf, LD, tw, load, emit);
+    fftp_lines<C, LEN, true, TC, NT, LAY_COL, false, false, false>(buf, LD, a.twF, load, emit);
 }
 
 template <typename T, int LEN>
@@ -1455,9 +1434,8 @@ __global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_inv_min_ctas<T, LE
     cols_inv_p_body<T, LEN>(a);
 }
 
-// Inverse x of rows of N points: the per-block argmax of the real part (ties to
-// the lowest index) or the complex map.
-template <typename T, int LEN, int MODE>
+// Inverse x of rows of N points: the complex map.
+template <typename T, int LEN>
 __device__ __forceinline__ void rows_inv_p_body(const RowArgs<T>& a) {
     using C = cplx<T>;
     constexpr int TR = lines_per_cta<T, LEN>();
@@ -1469,48 +1447,23 @@ __device__ __forceinline__ void rows_inv_p_body(const RowArgs<T>& a) {
     C* buf = reinterpret_cast<C*>(smem_raw);
     C* tw = buf + TR * LD;
     const int row0 = blockIdx.x * TR;
-    for (int j = threadIdx.x; j < NTW; j += blockDim.x) tw[j] = a.tw[j];
-    __syncthreads();
+    TwStage<C, NTW, cta_threads<T, LEN>()> tws;
+    tws.load(a.tw);
     const C* in = a.in + (int64_t)blockIdx.y * a.in_rot_stride + (int64_t)row0 * LEN;
+    C* out = a.out + (int64_t)blockIdx.y * a.out_rot_stride + (int64_t)row0 * LEN;
     const int nrows = a.nrows - row0;
     const C zero = mk(T(0), T(0));
     auto load = [&](int line, int i, int r) -> C { return line < nrows ? in[line * LEN + i + r * NB1] : zero; };
-    T best = -INFINITY;
-    int bidx = INT_MAX;
-    C* out = (MODE == ROW_INV_MAP) ? a.out + (int64_t)blockIdx.y * a.out_rot_stride + (int64_t)row0 * LEN : nullptr;
-    // one last-stage butterfly per thread: its outputs come in increasing index
-    // order, so a strict comparison already keeps the lowest index of equal values
-    constexpr bool one_bfly = TR * (LEN / plan_last_radix(LEN)) <= cta_threads<T, LEN>();
     auto emit = [&](int line, int i, int r, C v) {
-        if (line >= nrows) return;
-        if constexpr (MODE == ROW_INV_ARGMAX) {
-            if constexpr (one_bfly) {
-                if (v.x > best) {
-                    best = v.x;
-                    bidx = (row0 + line) * LEN + i + r * PL;
-                }
-            } else {
-                argmax_merge(best, bidx, v.x, (row0 + line) * LEN + i + r * PL);
-            }
-        } else {
-            out[line * LEN + i + r * PL] = v;
-        }
+        if (line < nrows) out[line * LEN + i + r * PL] = v;
     };
-    fftp_lines<C, LEN, true, TR, cta_threads<T, LEN>(), LAY_ROW, true, false, false>(buf, LD, tw, load, emit);
-    if constexpr (MODE == ROW_INV_ARGMAX) {
-        block_argmax(best, bidx);
-        if (threadIdx.x == 0) {
-            const int64_t o = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-            a.part_score[o] = (double)best;
-            a.part_idx[o] = bidx;
-        }
-    }
+    fftp_lines<C, LEN, true, TR, cta_threads<T, LEN>(), LAY_ROW, true, false, false>(buf, LD, tw, load, emit,
+                                                                                     LoadedHook([&] { tws.store(tw); }));
 }
 
-
-template <typename T, int LEN, int MODE>
+template <typename T, int LEN>
 __global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_inv_min_ctas<T, LEN>()) k_rows_inv_p(RowArgs<T> a) {
-    rows_inv_p_body<T, LEN, MODE>(a);
+    rows_inv_p_body<T, LEN>(a);
 }
 
 // ---------------------------------------------------------------------------
@@ -1594,51 +1547,6 @@ __global__ void __cluster_dims__(IYX_CS, 1, 1) __launch_bounds__(iyx_threads<T, 
             a.part_idx[o] = bidx;
         }
     }
-}
-
-// Inverse x of rows of N points keeping each block's K best translations of the
-// real part (score descending, index ascending): a sorted list per thread, merged
-// through shared memory after the transform; partials are K per block.
-template <typename T, int LEN, int K>
-__device__ __forceinline__ void rows_inv_topk_body(const RowArgs<T>& a) {
-    using C = cplx<T>;
-    constexpr int TR = lines_per_cta<T, LEN>();
-    constexpr int NT = cta_threads<T, LEN>();
-    constexpr int LD = line_pitch(LEN);
-    constexpr int NTW = tw_count(LEN);
-    constexpr int NB1 = LEN / plan_radix(LEN, 0);
-    constexpr int PL = LEN / plan_last_radix(LEN);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* buf = reinterpret_cast<C*>(smem_raw);
-    C* tw = buf + TR * LD;
-    T* sv = reinterpret_cast<T*>(tw + NTW);
-    int* si = reinterpret_cast<int*>(sv + NT * K);
-    __shared__ T wv[32], bestv[K];
-    __shared__ int wi[32], besti[K];
-    const int row0 = blockIdx.x * TR;
-    for (int j = threadIdx.x; j < NTW; j += blockDim.x) tw[j] = a.tw[j];
-    __syncthreads();
-    const C* in = a.in + (int64_t)blockIdx.y * a.in_rot_stride + (int64_t)row0 * LEN;
-    const int nrows = a.nrows - row0;
-    const C zero = mk(T(0), T(0));
-    auto load = [&](int line, int i, int r) -> C { return line < nrows ? in[line * LEN + i + r * NB1] : zero; };
-    TopK<T, K> top;
-    top.init();
-    auto emit = [&](int line, int i, int r, C v) {
-        if (line < nrows) top.push(v.x, (row0 + line) * LEN + i + r * PL);
-    };
-    fftp_lines<C, LEN, true, TR, NT, LAY_ROW, true, false, false>(buf, LD, tw, load, emit);
-    block_topk_merge<T, K>(top, sv, si, wv, wi, bestv, besti);
-    if (threadIdx.x < K) {
-        const int64_t o = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * K + threadIdx.x;
-        a.part_score[o] = (double)bestv[threadIdx.x];
-        a.part_idx[o] = besti[threadIdx.x];
-    }
-}
-
-template <typename T, int LEN, int K>
-__global__ void __launch_bounds__(cta_threads<T, LEN>()) k_rows_inv_topk(RowArgs<T> a) {
-    rows_inv_topk_body<T, LEN, K>(a);
 }
 
 // Resident CTAs per SM the pruned passes are compiled for (0: the compiler's choice).
@@ -1782,7 +1690,7 @@ static cudaError_t cols_fwd_p_launch(const ColArgs<T>& a, int batch, cudaStream_
     using C = cplx<T>;
     const int nb = (a.ncols + TC - 1) / TC;
     if (nb == 0 || batch == 0 || a.nouter == 0) return cudaSuccess;
-    const size_t smem = (size_t)(TC * col_pitch(LEN) + tw_count(LEN)) * sizeof(C);
+    const size_t smem = (size_t)TC * col_pitch(LEN) * sizeof(C);
     auto kern = k_cols_fwd_p<T, LEN, MB, TC>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
@@ -1835,16 +1743,16 @@ static cudaError_t cols_fused_p_impl(const ColArgs<T>& a, int batch, cudaStream_
     return cols_fused_p_launch<T, LENF, lines_per_cta<T, LENF>(), fused_std_min_ctas<T, LENF>()>(a, batch, st);
 }
 
-template <typename T, int LEN, int MODE>
+template <typename T, int LEN>
 static cudaError_t rows_inv_p_impl(const RowArgs<T>& a, int batch, int* nparts, cudaStream_t st) {
     using C = cplx<T>;
     constexpr int TR = lines_per_cta<T, LEN>();
     const int nb = (a.nrows + TR - 1) / TR;
     if (nparts) *nparts = nb;
     if (nb == 0 || batch == 0) return cudaSuccess;
-    if (a.in_row_stride != LEN || (MODE == ROW_INV_MAP && a.out_row_stride != LEN)) return cudaErrorInvalidValue;
+    if (a.in_row_stride != LEN || a.out_row_stride != LEN) return cudaErrorInvalidValue;
     const size_t smem = (size_t)(TR * line_pitch(LEN) + tw_count(LEN)) * sizeof(C);
-    auto kern = k_rows_inv_p<T, LEN, MODE>;
+    auto kern = k_rows_inv_p<T, LEN>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(nb, batch), cta_threads<T, LEN>(), smem, st>>>(a);
@@ -1898,7 +1806,7 @@ static cudaError_t cols_inv_p_impl(const ColArgs<T>& a, int batch, cudaStream_t 
     constexpr int TC = lines_per_cta<T, LEN>();
     const int nb = (a.ncols + TC - 1) / TC;
     if (nb == 0 || batch == 0 || a.nouter == 0) return cudaSuccess;
-    const size_t smem = (size_t)(TC * col_pitch(LEN) + tw_count(LEN)) * sizeof(C);
+    const size_t smem = (size_t)TC * col_pitch(LEN) * sizeof(C);
     auto kern = k_cols_inv_p<T, LEN>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
@@ -1907,48 +1815,12 @@ static cudaError_t cols_inv_p_impl(const ColArgs<T>& a, int batch, cudaStream_t 
     return cudaGetLastError();
 }
 
-template <typename T, int LEN, int K>
-static cudaError_t rows_inv_topk_impl(const RowArgs<T>& a, int batch, int* nparts, cudaStream_t st) {
-    using C = cplx<T>;
-    constexpr int TR = lines_per_cta<T, LEN>();
-    constexpr int NT = cta_threads<T, LEN>();
-    const int nb = (a.nrows + TR - 1) / TR;
-    if (nparts) *nparts = nb * K;
-    if (nb == 0 || batch == 0) return cudaSuccess;
-    if (a.in_row_stride != LEN) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)(TR * line_pitch(LEN) + tw_count(LEN)) * sizeof(C) + (size_t)NT * K * (sizeof(T) + sizeof(int));
-    auto kern = k_rows_inv_topk<T, LEN, K>;
-    cudaError_t e = set_smem(kern, smem);
-    if (e != cudaSuccess) return e;
-    kern<<<dim3(nb, batch), NT, smem, st>>>(a);
-    note_launch();
-    return cudaGetLastError();
-}
-
 template <typename T>
 cudaError_t launch_rows_t(int mode, const RowArgs<T>& a, int batch, int* nparts, cudaStream_t st) {
-    if (mode >= ROW_INV_TOPK2 && mode <= ROW_INV_TOPK16) {
+    if (mode == ROW_INV_MAP) {
         switch (a.N) {
-#define SD_ROWK_CASE(L)                                                                         \
-    case L:                                                                                     \
-        switch (mode) {                                                                         \
-            case ROW_INV_TOPK2: return rows_inv_topk_impl<T, L, 2>(a, batch, nparts, st);       \
-            case ROW_INV_TOPK4: return rows_inv_topk_impl<T, L, 4>(a, batch, nparts, st);       \
-            case ROW_INV_TOPK8: return rows_inv_topk_impl<T, L, 8>(a, batch, nparts, st);       \
-            default: return rows_inv_topk_impl<T, L, 16>(a, batch, nparts, st);                 \
-        }
-            SD_ROWK_CASE(8) SD_ROWK_CASE(16) SD_ROWK_CASE(24) SD_ROWK_CASE(32) SD_ROWK_CASE(48) SD_ROWK_CASE(64)
-            SD_ROWK_CASE(96) SD_ROWK_CASE(128) SD_ROWK_CASE(192) SD_ROWK_CASE(256)
-#undef SD_ROWK_CASE
-        }
-        return cudaErrorInvalidValue;
-    }
-    if (mode == ROW_INV_ARGMAX || mode == ROW_INV_MAP) {
-        switch (a.N) {
-#define SD_ROWI_CASE(L)                                                                                    \
-    case L:                                                                                                \
-        return mode == ROW_INV_ARGMAX ? rows_inv_p_impl<T, L, ROW_INV_ARGMAX>(a, batch, nparts, st)       \
-                                      : rows_inv_p_impl<T, L, ROW_INV_MAP>(a, batch, nparts, st);
+#define SD_ROWI_CASE(L) \
+    case L: return rows_inv_p_impl<T, L>(a, batch, nparts, st);
             SD_ROWI_CASE(8) SD_ROWI_CASE(16) SD_ROWI_CASE(24) SD_ROWI_CASE(32) SD_ROWI_CASE(48) SD_ROWI_CASE(64)
             SD_ROWI_CASE(96) SD_ROWI_CASE(128) SD_ROWI_CASE(192) SD_ROWI_CASE(256)
 #undef SD_ROWI_CASE
@@ -1965,17 +1837,14 @@ cudaError_t launch_rows_t(int mode, const RowArgs<T>& a, int batch, int* nparts,
         }
         return cudaErrorInvalidValue;
     }
-    const int len = (mode == ROW_FWD || mode == ROW_EXPAND) ? a.n : a.N;
 #define SD_ROW_CASE(L)                                                          \
     case L:                                                                     \
         switch (mode) {                                                         \
             case ROW_FWD: return rows_impl<T, L, ROW_FWD>(a, batch, nparts, st);   \
-            case ROW_INV_ARGMAX: return rows_impl<T, L, ROW_INV_ARGMAX>(a, batch, nparts, st); \
-            case ROW_INV_MAP: return rows_impl<T, L, ROW_INV_MAP>(a, batch, nparts, st); \
             case ROW_EXPAND: return rows_impl<T, L, ROW_EXPAND>(a, batch, nparts, st); \
         }                                                                       \
         break;
-    switch (len) { SD_FOR_EACH_LEN(SD_ROW_CASE) }
+    switch (a.n) { SD_FOR_EACH_LEN(SD_ROW_CASE) }
 #undef SD_ROW_CASE
     return cudaErrorInvalidValue;
 }
