@@ -1504,6 +1504,7 @@ static int sdf_build_t(sd_ctx* ctx, const void* bnd, const void* nrm, const void
     a.perm_q = perm_q;
     a.tile_box = ctx->opt_sdf_cull ? tbox : nullptr;
     a.sub_box = ctx->opt_sdf_cull >= 2 ? tbox + n_tiles * 6 : nullptr;
+    a.tree_box = tbox;
     a.n_tiles = n_tiles;
     e = launch_sdf<T>(a, ctx->p.dim, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1741,8 +1742,7 @@ int sd_score_pairs(sd_ctx* ctx, const sd_pair_job* jobs, int64_t n_jobs, sd_pair
 template <typename T>
 static int top_k_t(sd_ctx* ctx, const sd_cand* cand, int64_t n_cand, int k, int rescore, const sd_shape* fixed,
                    const sd_shape* moving, const double* quats, const sd_grid* g, sd_pose* out, cudaStream_t st) {
-    void *flags, *top, *res;
-    CKI(ws_get(ctx, 4, (size_t)((n_cand + 31) / 32) * 4 + 256, &flags));
+    void *top, *res;
     const size_t moved_bytes = rescore ? (size_t)k * moving->m * 4 * sizeof(double) : 0;
     const size_t box_bytes = rescore ? (size_t)k * rescore_tiles(moving->m) * 6 * sizeof(float) : 0;
     // layout: [top k sd_cand][re-scores 2k doubles][moved samples][tile boxes], 256-byte aligned
@@ -1753,7 +1753,7 @@ static int top_k_t(sd_ctx* ctx, const sd_cand* cand, int64_t n_cand, int k, int 
     res = (char*)top + res_off;
     void* moved = (char*)top + head;
     float* tile_box = (float*)((char*)moved + ((moved_bytes + 255) / 256) * 256);
-    CK(ctx, launch_topk(cand, n_cand, k, top, (unsigned*)flags, st));
+    CK(ctx, launch_topk(cand, n_cand, k, top, st));
     if (rescore) {
         RescoreArgs<T> a{};
         a.p1 = (const vec4<T>*)fixed->pos;

@@ -42,6 +42,7 @@ struct SdfArgs {
     const int32_t* perm_q;  // processing order of the queries (caller index), or null
     const float* tile_box;  // boundary tile boxes (n_tiles x 6: lo, hi), or null
     const float* sub_box;   // boxes of 32-sample sub-tiles (n_tiles * SDF_TILE / 32 x 6), or null
+    const float* tree_box;  // the boxes again, never null (3D): tiles, then sub-tiles
     int64_t n_tiles;        // boundary tiles of SDF_TILE samples
 };
 // Boundary samples gathered into Morton order: positions, normals with the
@@ -238,8 +239,8 @@ template <typename T>
 cudaError_t launch_interleave(const cplx<T>* src, cplx<T>* dst, int n, int pn, int dim, int f, cudaStream_t st);
 
 // ---- search -----------------------------------------------------------------
-cudaError_t launch_topk(const void* cand, int64_t n, int k, void* out_cand, unsigned* flags,
-                        cudaStream_t st);
+// The k best of n candidates, best first; no scratch memory.
+cudaError_t launch_topk(const void* cand, int64_t n, int k, void* out_cand, cudaStream_t st);
 template <typename T>
 struct RescoreArgs {
     const vec4<T>* p1; const cplx<T>* c1; int64_t m1;
