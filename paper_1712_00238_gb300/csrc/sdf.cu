@@ -210,31 +210,48 @@ __device__ __forceinline__ double4_32a load4(const double* p) { return *reinterp
 __device__ __forceinline__ float4 sample4(const float4* p) { return __ldg(p); }
 __device__ __forceinline__ double4_32a sample4(const double4_32a* p) { return *p; }
 
-// Winding sum, its dropped part's bound (over g) and the solid angles' magnitude of a far node.
-template <typename T>
-__device__ __forceinline__ void node_eval(const T* nd, const vec4<T>& p, T& wind, T& err, T& mag) {
+// Reciprocal square root; a denormal squared distance (coinciding points) counts as zero.
+__device__ __forceinline__ float rsqrt_(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
+
+// A far node's winding sum at the lane's Q points, its dropped part's bound (over g)
+// and its solid angle's magnitude.
+template <typename T, int Q>
+__device__ __forceinline__ void node_eval(const T* nd, const vec4<T> (&p)[Q], T (&wind)[Q], T (&err)[Q], T (&mag)[Q]) {
     const vec4<T> n0 = load4(nd), n1 = load4(nd + 4), n2 = load4(nd + 8), n3 = load4(nd + 12), n4 = load4(nd + 16),
                   n5 = load4(nd + 20), n6 = load4(nd + 24);
-    const T x = n0.x - p.x, y = n0.y - p.y, z = n0.z - p.z;
-    const T xx = x * x, yy = y * y, zz = z * z, xy = x * y, xz = x * z, yz = y * z;
-    const T ri = rsqrt(xx + yy + zz);
-    const T r2 = ri * ri, r3 = r2 * ri, r5 = r3 * r2;
-    const T Q = n2.x * xx + n2.y * yy + n2.z * zz + n2.w * xy + n3.x * xz + n3.y * yz;
-    const T VR = n3.w * x + n4.x * y + n4.y * z;
-    const T C = xx * (n4.z * x + n4.w * y + n5.x * z) + yy * (n5.y * x + n5.z * y + n5.w * z) +
-                zz * (n6.x * x + n6.y * y + n6.z * z) + xy * z * n6.w;
-    wind += r3 * (n1.x * x + n1.y * y + n1.z * z + (n2.x + n2.y + n2.z)) +
-            r5 * (T(7.5) * r2 * C - T(3) * Q - T(1.5) * VR);
-    err += n3.z * r5;
-    mag += n1.w * r2;
+    const T tr = n2.x + n2.y + n2.z;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const T x = n0.x - p[q].x, y = n0.y - p[q].y, z = n0.z - p[q].z;
+        const T xx = x * x, yy = y * y, zz = z * z, xy = x * y;
+        const T ri = rsqrt_(xx + yy + zz);
+        const T r2 = ri * ri, r3 = r2 * ri, r5 = r3 * r2;
+        const T M = n2.x * xx + n2.y * yy + n2.z * zz + n2.w * xy + z * (n3.x * x + n3.y * y);
+        const T VR = n3.w * x + n4.x * y + n4.y * z;
+        const T C = xx * (n4.z * x + n4.w * y + n5.x * z) + yy * (n5.y * x + n5.z * y + n5.w * z) +
+                    zz * (n6.x * x + n6.y * y + n6.z * z) + xy * z * n6.w;
+        wind[q] += r3 * (n1.x * x + n1.y * y + n1.z * z + tr) + r5 * (T(7.5) * r2 * C - T(3) * M - T(1.5) * VR);
+        err[q] += n3.z * r5;
+        mag[q] += n1.w * r2;
+    }
 }
 
 // The warp's box of query points (lo[3], hi[3]), in float, widened for the rounding.
-template <typename T>
-__device__ __forceinline__ void warp_box(const vec4<T>& p, float lo[3], float hi[3]) {
-    const float v[3] = {(float)p.x, (float)p.y, (float)p.z};
+template <typename T, int Q>
+__device__ __forceinline__ void warp_box(const vec4<T> (&p)[Q], float lo[3], float hi[3]) {
     for (int d = 0; d < 3; ++d) {
-        lo[d] = hi[d] = v[d];
+        lo[d] = INFINITY;
+        hi[d] = -INFINITY;
+        for (int q = 0; q < Q; ++q) {
+            const float v = (float)(d == 0 ? p[q].x : (d == 1 ? p[q].y : p[q].z));
+            lo[d] = fminf(lo[d], v);
+            hi[d] = fmaxf(hi[d], v);
+        }
         for (int off = 16; off > 0; off >>= 1) {
             lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], off));
             hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], off));
@@ -253,6 +270,20 @@ __device__ __forceinline__ float box_gap2(const float* b, const float lo[3], con
     }
     return g2;
 }
+// The same from one point: a warp whose 32 queries straddle a fold of the Morton
+// curve has a box full of nothing, so what its box lets through is put to a vote.
+template <typename T>
+__device__ __forceinline__ float point_gap2(const float* b, const vec4<T>& p) {
+    const float v[3] = {(float)p.x, (float)p.y, (float)p.z};
+    float g2 = 0.f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const float m = 1e-6f * (fabsf(v[d]) + 1.f);
+        const float g = fmaxf(0.f, fmaxf(b[d] - v[d], v[d] - b[3 + d]) - m);
+        g2 = fmaf(g, g, g2);
+    }
+    return g2;
+}
 // Whether a node is far enough from every point of the box for its expansion.
 template <typename T>
 __device__ __forceinline__ bool node_far(const T* nd, const float lo[3], const float hi[3]) {
@@ -267,25 +298,34 @@ __device__ __forceinline__ bool node_far(const T* nd, const float lo[3], const f
     return g2 >= need * need * 1.0001f;
 }
 
-// One CTA per 32 Morton-consecutive queries (one per lane of each of its 8 warps);
-// the warps share the tiles, lanes test 32 of them at a time, and each node or
-// sample that passes is evaluated by all lanes from broadcast loads.
+// One CTA per 32 Q Morton-consecutive queries (Q per lane of each of its 8 warps).
+// Lanes test 32 tiles at a time; the warps share the far tiles, and each takes one
+// of a near tile's 8 sub-tiles, so they finish together.  Nodes and samples are
+// broadcast loads, four wavefronts per 16 bytes: the L1 data pipe is what bounds the
+// kernel (88 % at one query a lane), and two queries a lane halve them.
 constexpr int TREE_NW = 8;
+// Two queries a lane where that still gives every SM two CTAs.
+constexpr int64_t TREE_PAIR_MIN = 64 * 2 * 152;
 
-template <typename T>
+template <typename T, int Q>
 __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T* nodes, const float* tile_box,
                                                            const float* sub_box, int* list, int* list_n) {
     constexpr int SUB = SDF_TILE / 32;
-    static_assert(SUB == TREE_NW, "the first tile's sub-tiles go to the warps");
-    __shared__ T sh[3][TREE_NW][32];
+    static_assert(SUB == TREE_NW, "a tile's sub-tiles go to the warps");
+    __shared__ T sh[3][TREE_NW][32 * Q];
     __shared__ float best_gap[TREE_NW];
     __shared__ int best_tile[TREE_NW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t i = min((int64_t)blockIdx.x * 32 + lane, a.m - 1);  // the last group's spare lanes repeat a query
-    const vec4<T> p = a.qry[a.perm_q ? (int64_t)a.perm_q[i] : i];
+    const int64_t i0 = (int64_t)blockIdx.x * (32 * Q) + lane;
+    vec4<T> p[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int64_t i = min(i0 + 32 * q, a.m - 1);  // the last group's spare places repeat a query
+        p[q] = a.qry[a.perm_q ? (int64_t)a.perm_q[i] : i];
+    }
     const int n_tiles = (int)a.n_tiles;
     float lo[3], hi[3];
-    warp_box<T>(p, lo, hi);
+    warp_box<T, Q>(p, lo, hi);
 
     // nearest sample: a first bound from the nearest tile
     float gap = INFINITY;
@@ -305,110 +345,138 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T
     tile0 = best_tile[0];
     for (int w = 1; w < TREE_NW; ++w)
         if (best_gap[w] < gap) { gap = best_gap[w]; tile0 = best_tile[w]; }
-    T dmin = INFINITY;
+    T dmin[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) dmin[q] = INFINITY;
     auto scan_sub = [&](int64_t j0) {  // the samples of one sub-tile
         const int cnt = (int)min((int64_t)32, a.n_b - j0);
-        const vec4<T>* q = a.bnd + j0;
+        const vec4<T>* b = a.bnd + j0;
 #pragma unroll 4
         for (int k = 0; k < cnt; ++k) {
-            const vec4<T> s = sample4(q + k);
-            const T dx = s.x - p.x, dy = s.y - p.y, dz = s.z - p.z;
-            const T d2 = dx * dx + dy * dy + dz * dz;
-            dmin = d2 < dmin ? d2 : dmin;
+            const vec4<T> s = sample4(b + k);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const T dx = s.x - p[q].x, dy = s.y - p[q].y, dz = s.z - p[q].z;
+                const T d2 = dx * dx + dy * dy + dz * dz;
+                dmin[q] = d2 < dmin[q] ? d2 : dmin[q];
+            }
         }
     };
     scan_sub((int64_t)tile0 * SDF_TILE + warp * 32);
-    sh[0][warp][lane] = dmin;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) sh[0][warp][lane + 32 * q] = dmin[q];
     __syncthreads();
-    for (int w = 0; w < TREE_NW; ++w) dmin = sh[0][w][lane] < dmin ? sh[0][w][lane] : dmin;
-    // every lane's nearest so far, with room for the rounding of the gaps
-    auto bound = [&] {
-        float b = (float)dmin;
-        for (int off = 16; off > 0; off >>= 1) b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, off));
-        return b * 1.00001f + 1e-30f;
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        for (int w = 0; w < TREE_NW; ++w) {
+            const T o = sh[0][w][lane + 32 * q];
+            dmin[q] = o < dmin[q] ? o : dmin[q];
+        }
+    // each query's nearest so far, with room for the rounding of the gaps, against a box
+    auto beyond = [&](const float* box) {
+        bool far = true;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) far &= point_gap2<T>(box, p[q]) > (float)dmin[q] * 1.00001f + 1e-30f;
+        return __all_sync(0xffffffffu, far);
     };
-    float ub = bound();
-    for (int base = 0; base < n_tiles; base += 32 * TREE_NW) {
-        const int t = base + lane * TREE_NW + warp;
-        const bool near = t < n_tiles && t != tile0 && !(box_gap2(tile_box + (int64_t)t * 6, lo, hi) > ub);
-        unsigned m = __ballot_sync(0xffffffffu, near);
+    float ub = 0.f;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) ub = fmaxf(ub, (float)dmin[q] * 1.00001f + 1e-30f);
+    for (int off = 16; off > 0; off >>= 1) ub = fmaxf(ub, __shfl_xor_sync(0xffffffffu, ub, off));
+    for (int base = 0; base < n_tiles; base += 32) {
+        const int t = base + lane;
+        unsigned m = __ballot_sync(0xffffffffu, t < n_tiles && t != tile0 &&
+                                                    !(box_gap2(tile_box + (int64_t)t * 6, lo, hi) > ub));
         while (m) {
-            const int tt = base + (__ffs(m) - 1) * TREE_NW + warp;
+            const int tt = base + __ffs(m) - 1;
             m &= m - 1;
-            const bool sn = lane < SUB && !(box_gap2(sub_box + ((int64_t)tt * SUB + (lane & (SUB - 1))) * 6, lo, hi) > ub);
-            unsigned ms = __ballot_sync(0xffffffffu, sn);
-            if (!ms) continue;
-            while (ms) {
-                scan_sub((int64_t)tt * SDF_TILE + (__ffs(ms) - 1) * 32);
-                ms &= ms - 1;
-            }
-            ub = bound();
+            if (!beyond(sub_box + ((int64_t)tt * SUB + warp) * 6)) scan_sub((int64_t)tt * SDF_TILE + warp * 32);
         }
     }
     __syncthreads();
-    sh[0][warp][lane] = dmin;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) sh[0][warp][lane + 32 * q] = dmin[q];
 
     // winding sum
-    T wind = T(0), err = T(0), mag = T(0);
+    T wind[Q], err[Q], mag[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) wind[q] = err[q] = mag[q] = T(0);
     if (!a.pmc_override) {
         const T* subs = nodes + (int64_t)n_tiles * NODE;
-        for (int base = 0; base < n_tiles; base += 32 * TREE_NW) {
-            const int t = base + lane * TREE_NW + warp;
+        auto all_far = [&](const T* nd) {
+            const vec4<T> c = load4(nd);
+            const T need = T(TREE_BETA) * c.w;
+            bool far = true;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const T dx = c.x - p[q].x, dy = c.y - p[q].y, dz = c.z - p[q].z;
+                far &= dx * dx + dy * dy + dz * dz >= need * need * T(1.0001);
+            }
+            return __all_sync(0xffffffffu, far);
+        };
+        for (int base = 0; base < n_tiles; base += 32) {
+            const int t = base + lane;
             const bool in = t < n_tiles;
             const bool far = in && node_far<T>(nodes + (int64_t)(in ? t : 0) * NODE, lo, hi);
-            unsigned mf = __ballot_sync(0xffffffffu, far), mn = __ballot_sync(0xffffffffu, in && !far);
+            // far tiles: dealt to the warps
+            unsigned mf = __ballot_sync(0xffffffffu, far) & (0x01010101u << warp);
+            unsigned mn = __ballot_sync(0xffffffffu, in && !far);
             while (mf) {
-                const int tt = base + (__ffs(mf) - 1) * TREE_NW + warp;
+                const int tt = base + __ffs(mf) - 1;
                 mf &= mf - 1;
-                node_eval<T>(nodes + (int64_t)tt * NODE, p, wind, err, mag);
+                node_eval<T, Q>(nodes + (int64_t)tt * NODE, p, wind, err, mag);
             }
             while (mn) {
-                const int tt = base + (__ffs(mn) - 1) * TREE_NW + warp;
+                const int tt = base + __ffs(mn) - 1;
                 mn &= mn - 1;
-                const T* sn = subs + (int64_t)tt * SUB * NODE;
-                const T* mine = sn + (lane & (SUB - 1)) * NODE;
-                const bool some = lane < SUB && !(mine[3] < T(0));
-                const bool sfar = some && node_far<T>(mine, lo, hi);
-                unsigned sf = __ballot_sync(0xffffffffu, sfar), sd = __ballot_sync(0xffffffffu, some && !sfar);
-                while (sf) {
-                    node_eval<T>(sn + (__ffs(sf) - 1) * NODE, p, wind, err, mag);
-                    sf &= sf - 1;
+                if (all_far(nodes + (int64_t)tt * NODE)) {  // the same in every warp
+                    if ((tt & (TREE_NW - 1)) == warp) node_eval<T, Q>(nodes + (int64_t)tt * NODE, p, wind, err, mag);
+                    continue;
                 }
-                while (sd) {
-                    const int64_t j0 = (int64_t)tt * SDF_TILE + (__ffs(sd) - 1) * 32;
-                    sd &= sd - 1;
-                    const int cnt = (int)min((int64_t)32, a.n_b - j0);
+                const T* nd = subs + ((int64_t)tt * SUB + warp) * NODE;
+                const int64_t j0 = (int64_t)tt * SDF_TILE + warp * 32;
+                const int cnt = (int)min((int64_t)32, a.n_b - j0);
+                if (cnt <= 0) continue;
+                if (all_far(nd)) {
+                    node_eval<T, Q>(nd, p, wind, err, mag);
+                    continue;
+                }
 #pragma unroll 4
-                    for (int k = 0; k < cnt; ++k) {
-                        const vec4<T> q = sample4(a.bnd + j0 + k), nn = sample4(a.nrm + j0 + k);
-                        const T dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
-                        const T r = rsqrt(dx * dx + dy * dy + dz * dz);
-                        wind += nn.w * (dx * nn.x + dy * nn.y + dz * nn.z) * r * r * r;
+                for (int k = 0; k < cnt; ++k) {
+                    const vec4<T> s = sample4(a.bnd + j0 + k), nn = sample4(a.nrm + j0 + k);
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) {
+                        const T dx = s.x - p[q].x, dy = s.y - p[q].y, dz = s.z - p[q].z;
+                        const T r = rsqrt_(dx * dx + dy * dy + dz * dz);
+                        wind[q] += nn.w * (dx * nn.x + dy * nn.y + dz * nn.z) * r * r * r;
                     }
                 }
             }
         }
     }
-    T* w0 = &sh[1][warp][lane];
-    *w0 = wind;
     constexpr float X = 1.f / TREE_BETA;
     constexpr float G = 4.f / (1.f - X) + X / ((1.f - X) * (1.f - X));
     constexpr double S = 4.0 * M_PI;
-    sh[2][warp][lane] = err * T(G * 1.001f) + mag * T(1e-4);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        sh[1][warp][lane + 32 * q] = wind[q];
+        sh[2][warp][lane + 32 * q] = err[q] * T(G * 1.001f) + mag[q] * T(1e-4);
+    }
     __syncthreads();
-    if (warp == 0 && (int64_t)blockIdx.x * 32 + lane < a.m) {
-        T e = T(0.01 * S);
-        wind = T(0);
+    const int64_t i = (int64_t)blockIdx.x * (32 * Q) + threadIdx.x;
+    if (threadIdx.x < 32 * Q && i < a.m) {
+        T d = INFINITY, e = T(0.01 * S), over = T(0);
         for (int w = 0; w < TREE_NW; ++w) {
-            dmin = sh[0][w][lane] < dmin ? sh[0][w][lane] : dmin;
-            wind += sh[1][w][lane];
-            e += sh[2][w][lane];
+            const T o = sh[0][w][threadIdx.x];
+            d = o < d ? o : d;
+            over += sh[1][w][threadIdx.x];
+            e += sh[2][w][threadIdx.x];
         }
-        a.xi_abs[i] = sqrt(dmin);
+        a.xi_abs[i] = sqrt(d);
         if (a.pmc_override) {
             a.pmc[i] = a.pmc_override[a.perm_q ? (int64_t)a.perm_q[i] : i] < 0 ? int8_t(-1) : int8_t(1);
         } else {
-            const T over = wind - T(0.5 * S);
+            over -= T(0.5 * S);
             a.pmc[i] = over > T(0) ? int8_t(-1) : int8_t(1);
             if (!(fabs(over) > e)) list[atomicAdd(list_n, 1)] = (int)i;  // undecided (or not a number)
         }
@@ -599,9 +667,9 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_sum(SdfArgs<T> a, int tiles_pe
 }
 
 // The same sum (3D, Eq. 15 with a truncation) over the tree: one CTA per 32
-// queries as in k_sdf_tree, each warp over its share of the tiles, testing them 32
-// at a time; a sub-tile beyond the warp's reach (1 + eps) max|xi| holds no pair that
-// passes Eq. 17t.  What a lane adds, and in which order, does not depend on what
+// queries as in k_sdf_tree, tiles tested 32 at a time against the warp's reach
+// (1 + eps) max|xi|, each warp taking one of a tile's sub-tiles unless it lies beyond
+// every lane's own reach: what is skipped holds no pair that passes Eq. 17t.  What a lane adds, and in which order, does not depend on what
 // is skipped.  (One CTA per 256 queries, in lock-step over whole tiles: 14.0 ms for
 // 5,000 spheres.)
 template <typename T>
@@ -615,11 +683,14 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_sum_tree(SdfArgs<T> a) {
     const T xabs = a.xi_abs[i];
     const T xi = a.pmc[i] < 0 ? -xabs : xabs;
     float lo[3], hi[3];
-    warp_box<T>(p, lo, hi);
+    const vec4<T> pp[1] = {p};
+    warp_box<T, 1>(pp, lo, hi);
     float reach = (float)xabs;
     for (int off = 16; off > 0; off >>= 1) reach = fmaxf(reach, __shfl_xor_sync(0xffffffffu, reach, off));
     reach = reach * (1.f + (float)a.eps) * (1.f + 1e-4f) + 1e-6f;
     const float reach2 = reach * reach;
+    const float own_reach = (float)xabs * (1.f + (float)a.eps) * (1.f + 1e-4f) + 1e-6f;
+    const float own2 = own_reach * own_reach;
     const T lam = xi > T(0) ? a.lam1 : -a.lam2;
     const T pref = lam / (T(2.0 * M_PI) * a.sigma);
     const T inv_xabs = recip(xabs);
@@ -627,40 +698,35 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_sum_tree(SdfArgs<T> a) {
     const T xi2 = xi * xi;
     T sr = 0, cr = 0, si = 0, ci = 0;
     const int n_tiles = (int)a.n_tiles;
-    for (int base = 0; base < n_tiles; base += 32 * TREE_NW) {
-        const int t = base + lane * TREE_NW + warp;
+    for (int base = 0; base < n_tiles; base += 32) {
+        const int t = base + lane;
         // NaN reach (a query whose distance is none) keeps every tile
         const bool in = t < n_tiles && !(a.tile_box && box_gap2(a.tile_box + (int64_t)t * 6, lo, hi) > reach2);
         unsigned m = __ballot_sync(0xffffffffu, in);
         while (m) {
-            const int tt = base + (__ffs(m) - 1) * TREE_NW + warp;
+            const int tt = base + __ffs(m) - 1;
             m &= m - 1;
-            const int64_t s0 = (int64_t)tt * SUB + (lane & (SUB - 1));
-            const bool sn = lane < SUB && s0 * 32 < a.n_b &&
-                            !(a.sub_box && box_gap2(a.sub_box + s0 * 6, lo, hi) > reach2);
-            unsigned ms = __ballot_sync(0xffffffffu, sn);
-            while (ms) {
-                const int64_t j0 = (int64_t)tt * SDF_TILE + (__ffs(ms) - 1) * 32;
-                ms &= ms - 1;
-                const int cnt = (int)min((int64_t)32, a.n_b - j0);
+            const int64_t j0 = (int64_t)tt * SDF_TILE + warp * 32;
+            const int cnt = (int)min((int64_t)32, a.n_b - j0);
+            if (a.sub_box && __all_sync(0xffffffffu, point_gap2<T>(a.sub_box + ((int64_t)tt * SUB + warp) * 6, p) > own2))
+                continue;
 #pragma unroll 2
-                for (int k = 0; k < cnt; ++k) {
-                    const vec4<T> q = sample4(a.bnd + j0 + k);
-                    const T dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
-                    const T d2 = dx * dx + dy * dy + dz * dz;
-                    const T eta = sqrt(d2);
-                    const T rm1 = eta * inv_xabs - T(1);
-                    if (rm1 > a.eps) continue;
-                    const vec4<T> nn = sample4(a.nrm + j0 + k);
-                    const T E = exp(-rm1 * rm1 * inv_2s2);
-                    const T cos_t = (dx * nn.x + dy * nn.y + dz * nn.z) * recip(eta);
-                    // zeta^-2 = (xi - i eta)^2 / (xi^2 + eta^2)^2
-                    const T den = xi2 + d2;
-                    const T inv_den2 = recip(den * den);
-                    const T f = pref * E * cos_t * nn.w;
-                    kahan_add(sr, cr, f * ((xi2 - d2) * inv_den2));
-                    kahan_add(si, ci, f * (T(-2) * xi * eta * inv_den2));
-                }
+            for (int k = 0; k < cnt; ++k) {
+                const vec4<T> q = sample4(a.bnd + j0 + k);
+                const T dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+                const T d2 = dx * dx + dy * dy + dz * dz;
+                const T eta = sqrt(d2);
+                const T rm1 = eta * inv_xabs - T(1);
+                if (rm1 > a.eps) continue;
+                const vec4<T> nn = sample4(a.nrm + j0 + k);
+                const T E = exp(-rm1 * rm1 * inv_2s2);
+                const T cos_t = (dx * nn.x + dy * nn.y + dz * nn.z) * recip(eta);
+                // zeta^-2 = (xi - i eta)^2 / (xi^2 + eta^2)^2
+                const T den = xi2 + d2;
+                const T inv_den2 = recip(den * den);
+                const T f = pref * E * cos_t * nn.w;
+                kahan_add(sr, cr, f * ((xi2 - d2) * inv_den2));
+                kahan_add(si, ci, f * (T(-2) * xi * eta * inv_den2));
             }
         }
     }
@@ -834,7 +900,10 @@ static cudaError_t launch_nearest(const SdfArgs<T>& a, int dim, cudaStream_t st)
             k_sdf_nodes<T><<<(unsigned)a.n_tiles, SDF_TILE, 0, st>>>(a.bnd, a.nrm, a.n_b, a.tree_box, sub_box, nodes, a.n_tiles);
             note_launch();
         }
-        k_sdf_tree<T><<<(unsigned)((a.m + 31) / 32), 32 * TREE_NW, 0, st>>>(a, nodes, a.tree_box, sub_box, list, list_n);
+        if (sizeof(T) == 4 && a.m >= TREE_PAIR_MIN)
+            k_sdf_tree<T, 2><<<(unsigned)((a.m + 63) / 64), 32 * TREE_NW, 0, st>>>(a, nodes, a.tree_box, sub_box, list, list_n);
+        else
+            k_sdf_tree<T, 1><<<(unsigned)((a.m + 31) / 32), 32 * TREE_NW, 0, st>>>(a, nodes, a.tree_box, sub_box, list, list_n);
         note_launch();
         if (!a.pmc_override) {
             k_sdf_wind_list<T><<<LIST_CTAS, SDF_TILE, 0, st>>>(a, list, list_n, part);
