@@ -282,7 +282,28 @@ __global__ void __launch_bounds__(RS_TILE) k_rescore_move(RescoreArgs<T> a) {
 // Pairs that pass the FP32 screen are queued per warp and evaluated 32 at a
 // time in FP64 with every lane busy: only the pose's total is needed, so any
 // lane may take any pair.
+// The FP64 pipe (1.06 TFLOP/s) bounds the kernel: 76 % busy over 21.6 ms at the
+// docking pair's top 100.  The exponential is evaluated with as few FP64 operations
+// as its accuracy allows, 8 instead of about 17: exp(-u) = 2^(-m / 256) e^(-f ln 2 / 256)
+// with u 256 / ln 2 = m + f, m an integer (its fraction bits index a table of
+// 2^(-i / 256) in shared memory, the rest goes into the exponent), |f| <= 1/2, and the
+// last factor's Taylor series to the fourth order (the next term is below 4e-17).
 constexpr int RS_QUEUE = 256;  // pair slots per warp
+constexpr int RS_EXP = 256;    // entries of the table
+
+// exp(-r2 / (2 s^2)) from r2 and k = 256 / (2 s^2 ln 2); 0 <= r2 k < 2^18.
+__device__ __forceinline__ double gauss_exp(double r2, double k, const double* tab) {
+    const double magic = 6755399441055744.0;  // 1.5 * 2^52: the low word receives round(x)
+    const double t = fma(r2, k, magic);
+    const int m = __double2loint(t);
+    const double f = fma(r2, k, magic - t);
+    static_assert(RS_EXP == 1 << 8, "");
+    constexpr double c = -0.6931471805599453094 / RS_EXP;
+    const double q = f * fma(f, fma(f, fma(f, c * c * c * c / 24.0, c * c * c / 6.0), c * c / 2.0), c);
+    const double w = tab[m & (RS_EXP - 1)];
+    const double e = __hiloint2double(__double2hiint(w) - ((m >> 8) << 20), __double2loint(w));
+    return fma(e, q, e);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(RS_TILE) k_rescore(RescoreArgs<T> a) {
@@ -294,6 +315,7 @@ __global__ void __launch_bounds__(RS_TILE) k_rescore(RescoreArgs<T> a) {
     __shared__ float blo[3], bhi[3];
     __shared__ float slo[RS_WARPS][3], shi[RS_WARPS][3];  // boxes of the 32-sample slices of a moving tile
     __shared__ double tv[3];
+    __shared__ double etab[RS_EXP];
     __shared__ int skip;
     const int pose = blockIdx.y;
     const Cand cd = reinterpret_cast<const Cand*>(a.top)[pose];
@@ -304,7 +326,7 @@ __global__ void __launch_bounds__(RS_TILE) k_rescore(RescoreArgs<T> a) {
         tv[0] = t3[0]; tv[1] = t3[1]; tv[2] = t3[2];
     }
     const double sg2 = 2.0 * a.sigma_g * a.sigma_g;  // (sigma_g sqrt 2)^2
-    const double inv_2sg2 = 1.0 / (2.0 * sg2);
+    const double kexp = RS_EXP / (2.0 * sg2 * 0.6931471805599453094);
     const double cut = 8.0 * sqrt(sg2);
     const float cut2f = (float)(cut * cut) * 1.001f;
     const double norm = (a.dim == 3) ? pow(2.0 * M_PI * sg2, -1.5) : 1.0 / (2.0 * M_PI * sg2);
@@ -348,6 +370,8 @@ __global__ void __launch_bounds__(RS_TILE) k_rescore(RescoreArgs<T> a) {
     }
     __syncthreads();
     if (skip) return;
+    static_assert(RS_EXP == RS_TILE, "one table entry per thread");
+    etab[threadIdx.x] = exp2(-(double)threadIdx.x / RS_EXP);  // visible after the first tile's barrier
     // tile test margin: float rounding of both boxes
     const double mag = fabs(tv[0]) + fabs(tv[1]) + fabs(tv[2]) + sqrt(a.r2max) + 1.0;
     const float cmarg = (float)(cut * (1.0 + 1e-4) + 1e-6 * mag);
@@ -366,7 +390,7 @@ __global__ void __launch_bounds__(RS_TILE) k_rescore(RescoreArgs<T> a) {
             if (q < upto) {
                 const int fi = queue[q][0], mj = queue[q][1];
                 const double dx = yx[mj] - qx1[fi], dy = yy[mj] - qy1[fi], dz = yz[mj] - qz1[fi];
-                const double g = norm * exp(-(dx * dx + dy * dy + dz * dz) * inv_2sg2);
+                const double g = gauss_exp(dx * dx + dy * dy + dz * dz, kexp, etab);
                 const double br = cr[mj] * g, bi = ci[mj] * g;
                 sr += ar1[fi] * br - ai1[fi] * bi;
                 si += ar1[fi] * bi + ai1[fi] * br;
@@ -449,8 +473,8 @@ __global__ void __launch_bounds__(RS_TILE) k_rescore(RescoreArgs<T> a) {
         si += __shfl_down_sync(0xffffffffu, si, off);
     }
     if (lane == 0) {
-        atomicAdd(a.out + 2 * pose, sr);
-        atomicAdd(a.out + 2 * pose + 1, si);
+        atomicAdd(a.out + 2 * pose, norm * sr);
+        atomicAdd(a.out + 2 * pose + 1, norm * si);
     }
 }
 
