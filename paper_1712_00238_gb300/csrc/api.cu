@@ -580,7 +580,8 @@ static int spread_x_bins(int s, int* nby, int* nbz) {
 static size_t bins_bytes_x(int s, int64_t m, int batch) {
     int nby, nbz;
     const int nbins = spread_x_bins(s, &nby, &nbz);
-    return ((size_t)batch * (3 * (size_t)nbins + 1) + 4 * (size_t)batch * (size_t)m) * sizeof(int);
+    return (((size_t)batch * (3 * (size_t)nbins + 1) + 3 * (size_t)batch * (size_t)m + 3) / 4 * 4 +
+            (size_t)batch * (size_t)m * SPREADX_REC) * sizeof(int);
 }
 static void bins_layout_x(void* p, int s, int64_t m, int batch, BinArgs* bn, int* nbz) {
     int nby;
@@ -599,9 +600,10 @@ static void bins_layout_x(void* p, int s, int64_t m, int batch, BinArgs* bn, int
     q += (size_t)batch * m;
     bn->rank = q;
     q += (size_t)batch * m;
-    bn->sorted = q;
-    q += (size_t)batch * m;
+    bn->sorted = nullptr;
     bn->org = q;
+    q += (size_t)batch * m;
+    bn->rec = (float*)((int*)p + (q - (int*)p + 3) / 4 * 4);  // 16-byte aligned
 }
 
 // Binned spreading exists for FP32 and kernel widths 4-7 (tiles of tb + w - 1 cells).

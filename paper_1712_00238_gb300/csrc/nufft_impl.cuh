@@ -131,11 +131,47 @@ __device__ __forceinline__ void spread_row(cplx<T>* row, int s, int ax0, bool wr
     }
 }
 
+// The spreading kernel psi at z, from z^2: exp(beta (sqrt(1 - z^2) - 1)) for |z| <= 1,
+// else 0.  FP64 (64 rotations x 3,500 samples of the 2D workload are 2.7 million of
+// them, and the FP64 pipe does 1.06 TFLOP/s) takes about 20 FP64 operations: the
+// square root from an FP32 reciprocal root by one Newton step and one residual
+// correction, the exponential after Cody and Waite's reduction by multiples of
+// ln 2 / 64 (tab: 2^(-i / 64), i < 64; fifth-order series, next term below 4e-17).
+constexpr int ES_TAB = 64;
+__device__ __forceinline__ float es_weight(float z2, float beta, const double*) {
+    return (z2 <= 1.f) ? exp(beta * (sqrt(1.f - z2) - 1.f)) : 0.f;
+}
+__device__ __forceinline__ double es_weight(double z2, double beta, const double* tab) {
+    if (!(z2 <= 1.0)) return 0.0;
+    const double s = 1.0 - z2;
+    const double y0 = (double)rsqrtf(fmaxf((float)s, 1e-30f));
+    const double y1 = fma(0.5 * y0, fma(-s * y0, y0, 1.0), y0);
+    const double g = s * y1;
+    const double u = fma(fma(-g, g, s), 0.5 * y1, g);  // sqrt(s)
+    const double x = beta * (u - 1.0);                 // <= 0
+    if (x < -700.0) return 0.0;                        // below 1e-304
+    const double magic = 6755399441055744.0;           // 1.5 * 2^52: the low word receives round(.)
+    const double t = fma(x, ES_TAB * 1.4426950408889634074, magic);
+    const int m = -__double2loint(t);
+    const double k = t - magic;
+    constexpr double hi = 0x1.62e42fefap-1 / ES_TAB, lo = 0x1.cf79abc9e3b39p-40 / ES_TAB;  // ln 2 = hi + lo
+    const double r = fma(-k, lo, fma(-k, hi, x));
+    const double q = r * fma(r, fma(r, fma(r, fma(r, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), 0.5), 1.0);
+    const double w = tab[m & (ES_TAB - 1)];
+    const double e = __hiloint2double(__double2hiint(w) - ((m / ES_TAB) << 20), __double2loint(w));
+    return fma(e, q, e);
+}
+// Fills the table (double only); a barrier follows in the caller.
+template <typename T>
+__device__ __forceinline__ void es_table(double* tab) {
+    if (sizeof(T) == 8 && threadIdx.x < ES_TAB) tab[threadIdx.x] = exp2(-(double)threadIdx.x / ES_TAB);
+}
+
 // Taps of one sample: x/y weights in registers (unrolled loops), the z loop
 // rolled with its weight evaluated per iteration (no run-time-indexed arrays).
 template <typename T, int D, int W>
 __device__ __forceinline__ void spread_direct(cplx<T>* out, int s, int s_h, const int* u0, const T (*wt)[W],
-                                              cplx<T> c, T gz, T beta) {
+                                              cplx<T> c, T gz, T beta, const double* tab) {
     using C = cplx<T>;
     int ax0 = u0[0] + s_h;
     const bool wraps = (ax0 < 0) || (ax0 + W > s);
@@ -153,9 +189,7 @@ __device__ __forceinline__ void spread_direct(cplx<T>* out, int s, int s_h, cons
 #pragma unroll 1
         for (int kz = 0; kz < W; ++kz) {
             const T zz = (T(uz0 + kz) - gz) * inv_half;
-            const T z2 = zz * zz;
-            const T wz = (z2 <= T(1)) ? exp(beta * (sqrt(T(1) - z2) - T(1))) : T(0);
-            const C cz = cscale(c, wz);
+            const C cz = cscale(c, es_weight(zz * zz, beta, tab));
             C* plane = out + (int64_t)wrap_index(uz0 + kz + s_h, s) * s * s;
 #pragma unroll
             for (int ky = 0; ky < W; ++ky)
@@ -179,8 +213,10 @@ template <typename T, int D, int W>
 __global__ void __launch_bounds__(256) k_spread(SpreadArgs<T> a) {
     using C = cplx<T>;
     __shared__ T Rm[9];
+    __shared__ double etab[sizeof(T) == 8 ? ES_TAB : 1];
     const int b = blockIdx.y;
     if (threadIdx.x == 0) load_rotation(a, b, Rm);
+    es_table<T>(etab);
     __syncthreads();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= a.m) return;
@@ -201,13 +237,63 @@ __global__ void __launch_bounds__(256) k_spread(SpreadArgs<T> a) {
 #pragma unroll
         for (int k = 0; k < W; ++k) {
             const T z = (T(u0[d] + k) - g) * inv_half;
-            const T z2 = z * z;
-            wt[d][k] = (z2 <= T(1)) ? exp(a.beta * (sqrt(T(1) - z2) - T(1))) : T(0);
+            wt[d][k] = es_weight(z * z, a.beta, etab);
         }
     }
     const T gz = y[2] * a.inv_h;
     if (D == 3) u0[2] = (int)ceil(gz - half);
-    spread_direct<T, D, W>(a.out + (int64_t)b * a.out_rot_stride, a.s, a.s_h, u0, wt, c, gz, a.beta);
+    spread_direct<T, D, W>(a.out + (int64_t)b * a.out_rot_stride, a.s, a.s_h, u0, wt, c, gz, a.beta, etab);
+}
+
+// The same with eight lanes per sample, for launches too small to fill the GPU with
+// one thread each: lane k evaluates the k-th weight of every axis, the x (and in
+// 3D y) weights go round by shuffles, and the lane adds the k-th plane (2D: row) of
+// the tap box.
+template <typename T, int D, int W>
+__global__ void __launch_bounds__(256) k_spread_lanes(SpreadArgs<T> a) {
+    using C = cplx<T>;
+    static_assert(W <= 8, "a lane per plane");
+    __shared__ T Rm[9];
+    __shared__ double etab[sizeof(T) == 8 ? ES_TAB : 1];
+    const int b = blockIdx.y;
+    if (threadIdx.x == 0) load_rotation(a, b, Rm);
+    es_table<T>(etab);
+    __syncthreads();
+    const int64_t j = (int64_t)blockIdx.x * (blockDim.x / 8) + (threadIdx.x >> 3);
+    const bool live = j < a.m;
+    const int k = threadIdx.x & 7, first = threadIdx.x & 24;
+    const vec4<T> p = a.pos[live ? j : 0];
+    const C c = a.c[live ? j : 0];
+    const T half = T(W) * T(0.5), inv_half = T(2) / T(W);
+    T own[D];
+    int u0[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        const T g = a.sign * (Rm[3 * d] * p.x + Rm[3 * d + 1] * p.y + Rm[3 * d + 2] * p.z) * a.inv_h;
+        u0[d] = (int)ceil(g - half);
+        const T z = (T(u0[d] + k) - g) * inv_half;
+        own[d] = es_weight(z * z, a.beta, etab);
+    }
+    T wx[W], wy[W];
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+        wx[q] = __shfl_sync(0xffffffffu, own[0], first + q);
+        wy[q] = D == 3 ? __shfl_sync(0xffffffffu, own[1], first + q) : T(0);
+    }
+    if (!live || k >= W) return;
+    const int s = a.s;
+    int ax0 = u0[0] + a.s_h;
+    const bool wraps = (ax0 < 0) || (ax0 + W > s);
+    ax0 = wrap_index(ax0, s);
+    const C cl = cscale(c, own[D - 1]);
+    C* out = a.out + (int64_t)b * a.out_rot_stride + (int64_t)wrap_index(u0[D - 1] + k + a.s_h, s) * (D == 3 ? s * s : s);
+    if constexpr (D == 2) {
+        spread_row<T, W>(out, s, ax0, wraps, cl, wx);
+    } else {
+#pragma unroll
+        for (int ky = 0; ky < W; ++ky)
+            spread_row<T, W>(out + (int64_t)wrap_index(u0[1] + ky + a.s_h, s) * s, s, ax0, wraps, cscale(cl, wy[ky]), wx);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -849,13 +935,17 @@ __global__ void __launch_bounds__(BOX_SPC) k_spread_box(SpreadArgs<float> a) {
 // shared tile, then runs the pruned forward x transform of its rows straight
 // from the tile and writes the N kept modes of each row.  No sub-box is stored,
 // cleared or re-read, and no global atomic is issued.
+// A sample meets 3.4 CTAs on average, so its 18 kernel weights are evaluated once,
+// by the pass that sorts (k_records, 96 bytes a sample): a warp of the accumulation
+// reads a record with one load, lane by lane, a sample ahead, and deals it out by
+// shuffles, with no staging in shared memory and no barrier.
 
-constexpr int SX_W = 6, SX_TY = SPREADX_TY, SX_TZ = SPREADX_TZ, SX_TR = 6, SX_NT = 256, SX_CHUNK = 64;
+constexpr int SX_W = 6, SX_TY = SPREADX_TY, SX_TZ = SPREADX_TZ, SX_TR = 6, SX_NT = 256;
 static_assert(SX_TY >= SX_W - 1 && SX_TZ >= SX_W - 1, "a tap box must meet at most two bins per axis");
 static_assert((SX_TY * SX_TZ) % SX_TR == 0, "rows per FFT group must divide the rows of a bin");
-// staged record: w[axis][W] | origin[3] | c * scale (pair)
-constexpr int SX_O_ORG = 3 * SX_W, SX_O_C = 3 * SX_W + 4;
-constexpr int SX_REC = SX_O_C + 2;
+// record of a sample: w[axis][W] | packed origin | c (pair) | pad
+constexpr int SX_REC = SPREADX_REC, SX_O_ORG = 3 * SX_W, SX_O_C = 3 * SX_W + 1;
+static_assert(SX_O_C + 2 <= SX_REC && SX_REC <= 32, "a lane per entry of a record");
 
 // Row pitch of the shared tile (cells): at least s and 6 mod 32, so that the
 // lanes of a warp on consecutive taps of one tap box (x fastest) fall in
@@ -864,11 +954,7 @@ __host__ __device__ inline int spread_x_pitch(int s) { return s + ((6 - s % 32) 
 
 template <int LEN>
 __host__ __device__ constexpr size_t spread_x_smem_fixed() {
-    // twiddles + the larger of the staging records and the FFT line buffer
-    return (size_t)tw_count(LEN) * sizeof(float2) +
-           ((size_t)SX_CHUNK * SX_REC * sizeof(float) > (size_t)SX_TR * line_pitch(LEN) * sizeof(float2)
-                ? (size_t)SX_CHUNK * SX_REC * sizeof(float)
-                : (size_t)SX_TR * line_pitch(LEN) * sizeof(float2));
+    return (size_t)(tw_count(LEN) + SX_TR * line_pitch(LEN)) * sizeof(float2);  // twiddles, FFT line buffer
 }
 __host__ inline size_t spread_x_smem(int len, int px) {
     size_t fixed = 0;
@@ -908,10 +994,45 @@ __global__ void __launch_bounds__(256) k_bin_count_yz(SpreadArgs<T> a, BinArgs b
     }
 }
 
+// Sorted sample records of the fused spreading: four threads per sample, one axis's
+// weights each (about the origin the binning pass used), the fourth the origin and c.
+static __global__ void __launch_bounds__(256) k_records(SpreadArgs<float> a, BinArgs bn) {
+    __shared__ float Rm[9];
+    const int b = blockIdx.y;
+    if (threadIdx.x == 0) load_rotation(a, b, Rm);
+    __syncthreads();
+    const int64_t j = (int64_t)blockIdx.x * 64 + (threadIdx.x >> 2);
+    const int part = threadIdx.x & 3;
+    if (j >= a.m) return;
+    const int64_t o = (int64_t)b * a.m + j;
+    const int pos = bn.offset[(int64_t)b * (bn.nbins + 1) + bn.bin_of[o]] + bn.rank[o];
+    float* r = bn.rec + ((int64_t)b * a.m + pos) * SX_REC;
+    const int packed = bn.org[o];
+    if (part == 3) {
+        const float2 c = a.c[j];
+        r[SX_O_ORG] = __int_as_float(packed);
+        r[SX_O_C] = c.x;
+        r[SX_O_C + 1] = c.y;
+        return;
+    }
+    const float4 p = a.pos[j];
+    const float y = a.sign * (Rm[3 * part] * p.x + Rm[3 * part + 1] * p.y + Rm[3 * part + 2] * p.z);
+    const float g = y * a.inv_h;
+    const int u0 = ((packed >> (10 * part)) & 1023) - a.s_h;
+    float w[SX_W];
+#pragma unroll
+    for (int q = 0; q < SX_W; ++q) {
+        const float zz = ((float)(u0 + q) - g) * (2.f / SX_W);
+        w[q] = es_weight(zz * zz, a.beta, nullptr);
+    }
+#pragma unroll
+    for (int q = 0; q < SX_W; q += 2) *reinterpret_cast<float2*>(r + part * SX_W + q) = make_float2(w[q], w[q + 1]);
+}
+
 template <int LEN>
 __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinArgs bn, int nbz, int px,
                                                        float2* out, int64_t out_rot_stride, const float2* twg) {
-    constexpr int W = SX_W, TY = SX_TY, TZ = SX_TZ, TR = SX_TR, NT = SX_NT, CHUNK = SX_CHUNK, REC = SX_REC;
+    constexpr int W = SX_W, TY = SX_TY, TZ = SX_TZ, TR = SX_TR, NT = SX_NT;
     constexpr int ROWS = TY * TZ;
     constexpr int LD = line_pitch(LEN);
     constexpr int NTW = tw_count(LEN);
@@ -924,9 +1045,7 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
     int* tre = reinterpret_cast<int*>(sx_raw);
     int* tim = tre + ROWS * px;
     float2* tw = reinterpret_cast<float2*>(tim + ROWS * px);
-    float* stage = reinterpret_cast<float*>(tw + NTW);
-    float2* buf = reinterpret_cast<float2*>(tw + NTW);  // the same memory, after the accumulation
-    __shared__ float Rm[9];
+    float2* buf = tw + NTW;
     __shared__ unsigned char divtab[7][W * W];  // (rho / ny) << 4 | rho % ny
     const int b = blockIdx.y;
     const int nby = bn.nb;
@@ -934,34 +1053,31 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
     const int y0 = by * TY, z0 = bz * TZ;
     const int s = a.s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < ROWS * px; i += NT) {
-        tre[i] = 0;
-        tim[i] = 0;
-    }
-    for (int j = tid; j < NTW; j += NT) tw[j] = twg[j];
-    for (int i = tid; i < 7 * W * W; i += NT) {
-        const int ny = i / (W * W), rho = i % (W * W);
-        divtab[ny][rho] = ny ? (unsigned char)(((rho / ny) << 4) | (rho % ny)) : 0;
-    }
-    if (tid == 0) load_rotation(a, b, Rm);
-    // the source bins (by - {0, 1}) x (bz - {0, 1}) and their sample ranges
+    float2* outb = out + (int64_t)b * out_rot_stride;
+    // the source bins (by - {0, 1}) x (bz - {0, 1}): two runs of sorted samples
+    // (neighbours along y are adjacent), and a bound on the tile's cells: taps below
+    // 2^21, a cell's sum (at most the sum of |c|, the weights being <= 1) below 2^30;
+    // each bin's count times its largest |component| of c (from the binning pass)
+    // bounds that sum
     const int* off = bn.offset + (int64_t)b * (bn.nbins + 1);
-    __shared__ int src_lo[4], src_hi[4];
-    __shared__ float src_max[4];
-    if (tid < 4) {
-        const int yy = by - (tid & 1), zz = bz - (tid >> 1);
-        src_lo[tid] = src_hi[tid] = 0;
-        src_max[tid] = 0.f;
-        if (yy >= 0 && zz >= 0) {
-            src_lo[tid] = off[zz * nby + yy];
-            src_hi[tid] = off[zz * nby + yy + 1];
-            src_max[tid] = __int_as_float(bn.cmax[(int64_t)b * bn.nbins + zz * nby + yy]);
+    const int* cmax = bn.cmax + (int64_t)b * bn.nbins;
+    int run_lo[2] = {0, 0}, run_n[2] = {0, 0};
+    float mx = 0.f, sm = 0.f;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int zz = bz - k;
+        if (zz < 0) continue;
+        const int first = zz * nby + max(by - 1, 0), last = zz * nby + by;
+        run_lo[k] = off[first];
+        run_n[k] = off[last + 1] - run_lo[k];
+        for (int i = first; i <= last; ++i) {
+            const float cm = __int_as_float(cmax[i]);
+            mx = fmaxf(mx, cm);
+            sm += (float)(off[i + 1] - off[i]) * cm;
         }
     }
-    __syncthreads();
-    const int32_t* sorted = bn.sorted + (int64_t)b * a.m;
-    float2* outb = out + (int64_t)b * out_rot_stride;
-    if (src_hi[0] - src_lo[0] + src_hi[1] - src_lo[1] + src_hi[2] - src_lo[2] + src_hi[3] - src_lo[3] == 0) {
+    const int total = run_n[0] + run_n[1];
+    if (total == 0) {
         // no sample reaches these rows: their modes are zero
         for (int i = tid; i < ROWS * (NH / 2); i += NT) {
             const int l = i / (NH / 2), k = i % (NH / 2);
@@ -971,90 +1087,70 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
         }
         return;
     }
-    // fixed point: taps below 2^21, a cell's sum (at most the sum of |c| over the
-    // source samples, the weights being <= 1) below 2^30; each source bin's count
-    // times its largest |component| of c (from the binning pass) bounds that sum
-    float mx = 0.f, sm = 0.f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        mx = fmaxf(mx, src_max[k]);
-        sm += (float)(src_hi[k] - src_lo[k]) * src_max[k];
-    }
     const float scale = tile_scale(mx, sm * 1.0001f);
     const float inv_scale = 1.f / scale;  // a power of two: exact
-    // this lane's tap in each round of a full tap box: x tap and row (ky + ny kz flattened)
-    constexpr int ROUNDS = (W * W * W + 31) / 32;
-    int kx_of[ROUNDS], rho_of[ROUNDS];
-#pragma unroll
-    for (int q = 0; q < ROUNDS; ++q) {
-        const int tap = min(q * 32 + lane, W * W * W - 1);
-        kx_of[q] = tap % W;
-        rho_of[q] = tap / W;
+    // entry `lane` of record t of the runs
+    const float* recs = bn.rec + (int64_t)b * a.m * SX_REC + min(lane, SX_REC - 1);
+    auto fetch = [&](int t) -> float {
+        if (t >= total) return 0.f;
+        return recs[(int64_t)(t < run_n[0] ? run_lo[0] + t : run_lo[1] + t - run_n[0]) * SX_REC];
+    };
+    float next = fetch(warp);
+    for (int i = tid; i < ROWS * px / 2; i += NT) reinterpret_cast<int4*>(tre)[i] = make_int4(0, 0, 0, 0);
+    for (int j = tid; j < NTW; j += NT) tw[j] = twg[j];
+    for (int i = tid; i < 7 * W * W; i += NT) {
+        const int ny = i / (W * W), rho = i % (W * W);
+        divtab[ny][rho] = ny ? (unsigned char)(((rho / ny) << 4) | (rho % ny)) : 0;
     }
-#pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
-        for (int p0 = src_lo[k]; p0 < src_hi[k]; p0 += CHUNK) {
-            const int nj = min(CHUNK, src_hi[k] - p0);
-            // four threads per sample: the kernel weights of one axis each, and c
-            {
-                const int j = tid >> 2, part = tid & 3;
-                if (j < nj) {
-                    const int64_t js = sorted[p0 + j];
-                    float* r = stage + j * REC;
-                    if (part < 3) {
-                        // the origin the binning pass used, and the weights about it
-                        const int o = (bn.org[(int64_t)b * a.m + js] >> (10 * part)) & 1023;
-                        const float4 p = a.pos[js];
-                        const float y = a.sign * (Rm[3 * part] * p.x + Rm[3 * part + 1] * p.y + Rm[3 * part + 2] * p.z);
-                        const float g = y * a.inv_h;
-                        const int u0 = o - a.s_h;
+    __syncthreads();
+    // The warps take the samples in turn.  Lanes 0-29 hold five rows of six x taps a
+    // round; lane l also holds row l of the clipped tap box (weight wy wz, tile
+    // offset; rows 32-35 in a second pair) for the shuffles that deal rows out.
+    const int kx = lane % W, slot = lane / W;
+    const bool tap = lane < 5 * W;
+    for (int t = warp; t < total; t += NWARP) {
+        const float rec = next;
+        next = fetch(t + NWARP);
+        const int packed = __float_as_int(__shfl_sync(0xffffffffu, rec, SX_O_ORG));
+        const float cx = __shfl_sync(0xffffffffu, rec, SX_O_C) * scale, cy = __shfl_sync(0xffffffffu, rec, SX_O_C + 1) * scale;
+        const float wx = __shfl_sync(0xffffffffu, rec, kx);
+        const int dy = ((packed >> 10) & 1023) - y0, dz = (packed >> 20) - z0;
+        const int ly = max(0, -dy), hy = min(W, TY - dy);
+        const int lz = max(0, -dz), hz = min(W, TZ - dz);
+        const int ny = hy - ly, nz = hz - lz;
+        if (ny <= 0 || nz <= 0) continue;  // uniform over the warp
+        const int rows = ny * nz;
+        const int base = ((dz + lz) * TY + dy + ly) * px + (packed & 1023) + kx;
+        float row_w[2];
+        int row_o[2];
 #pragma unroll
-                        for (int q = 0; q < W; ++q) {
-                            const float zz = ((float)(u0 + q) - g) * (2.f / W);
-                            const float z2 = zz * zz;
-                            r[part * W + q] = (z2 <= 1.f) ? exp(a.beta * (sqrt(1.f - z2) - 1.f)) : 0.f;
-                        }
-                        r[SX_O_ORG + part] = __int_as_float(o);
-                    } else {
-                        const float2 c = a.c[js];
-                        r[SX_O_C] = c.x * scale;
-                        r[SX_O_C + 1] = c.y * scale;
-                    }
-                }
-            }
-            __syncthreads();
-            // the warps add the staged samples round-robin, lanes on consecutive taps
-            // of the sample's tap box clipped to this CTA's rows
-            for (int j = warp; j < nj; j += NWARP) {
-                const float* r = stage + j * REC;
-                const int ox = __float_as_int(r[SX_O_ORG]);
-                const int oy = __float_as_int(r[SX_O_ORG + 1]);
-                const int oz = __float_as_int(r[SX_O_ORG + 2]);
-                const int ly = max(0, y0 - oy), hy = min(W, y0 + TY - oy);
-                const int lz = max(0, z0 - oz), hz = min(W, z0 + TZ - oz);
-                const int ny = hy - ly, nz = hz - lz;
-                if (ny <= 0 || nz <= 0) continue;  // uniform over the warp
-                const int ntaps = W * ny * nz;
-                const int base = ((oz + lz - z0) * TY + (oy + ly - y0)) * px + ox;
-                const float cx = r[SX_O_C], cy = r[SX_O_C + 1];
-                const unsigned char* dv = divtab[ny];
+        for (int h = 0; h < 2; ++h) {
+            const int d = divtab[ny][h ? 32 + (lane & 3) : lane];
+            const int ry = d & 15, rz = d >> 4;
+            row_w[h] = __shfl_sync(0xffffffffu, rec, W + ly + ry) * __shfl_sync(0xffffffffu, rec, (2 * W + lz + rz) & 31);
+            row_o[h] = (rz * TY + ry) * px;
+            if (rows <= 32) break;  // uniform
+        }
 #pragma unroll
-                for (int q = 0; q < ROUNDS; ++q) {
-                    if (q * 32 >= ntaps) break;  // uniform over the warp
-                    if (q * 32 + lane < ntaps) {
-                        const int d = dv[rho_of[q]];
-                        const int ky = d & 15, kz = d >> 4;
-                        const int kx = kx_of[q];
-                        const int cell = base + kx + (kz * TY + ky) * px;
-                        const float w = r[kx] * r[W + ly + ky] * r[2 * W + lz + kz];
-                        atomicAdd(tre + cell, __float_as_int(fmaf(cx, w, MAGIC)) - MAGIC_BITS);
-                        atomicAdd(tim + cell, __float_as_int(fmaf(cy, w, MAGIC)) - MAGIC_BITS);
-                    }
-                }
+        for (int q = 0; q < 8; ++q) {
+            if (q * 5 >= rows) break;  // uniform
+            const int rr = q * 5 + slot;
+            float w = __shfl_sync(0xffffffffu, row_w[0], rr & 31);
+            int o = __shfl_sync(0xffffffffu, row_o[0], rr & 31);
+            if (q >= 6) {  // rows 30 on
+                const float w1 = __shfl_sync(0xffffffffu, row_w[1], rr & 3);
+                const int o1 = __shfl_sync(0xffffffffu, row_o[1], rr & 3);
+                if (rr >= 32) { w = w1; o = o1; }
             }
-            __syncthreads();  // the stage is refilled by the next chunk
+            if (tap && rr < rows) {
+                w *= wx;
+                const int cell = base + o;
+                atomicAdd(tre + cell, __float_as_int(fmaf(cx, w, MAGIC)) - MAGIC_BITS);
+                atomicAdd(tim + cell, __float_as_int(fmaf(cy, w, MAGIC)) - MAGIC_BITS);
+            }
         }
     }
+    __syncthreads();
     // forward x transform of the rows, TR at a time (row l: y = y0 + l % TY, z = z0 + l / TY)
     const float2 zero = make_float2(0.f, 0.f);
 #pragma unroll 1
@@ -1896,10 +1992,26 @@ cudaError_t launch_cols_t(int mode, const ColArgs<T>& a, int batch, cudaStream_t
     return cudaErrorInvalidValue;
 }
 
+// Samples in a launch up to which direct spreading takes eight lanes per sample: 12
+// rotations of 1,500 samples 28 -> 23 us, 13 of 2,280 29 -> 28; 64 of 2,280 (146 thousand)
+// are bound by the L2 atomics either way.
+constexpr int64_t SPREAD_LANES_MAX = 65536;
+
 template <typename T>
 cudaError_t launch_spread_t(const SpreadArgs<T>& a, int dim, int batch, cudaStream_t st) {
     if (a.m == 0 || batch == 0) return cudaSuccess;
     const dim3 grid((unsigned)((a.m + 255) / 256), batch);
+    const dim3 grid8((unsigned)((a.m + 31) / 32), batch);
+    const bool lanes = a.m * batch <= SPREAD_LANES_MAX;
+#define SD_SPREAD_LANES(WW)                                                                  \
+    if (lanes && a.w == WW) {                                                                \
+        auto kern = (dim == 2) ? k_spread_lanes<T, 2, WW> : k_spread_lanes<T, 3, WW>;        \
+        kern<<<grid8, 256, 0, st>>>(a);                                                      \
+        note_launch();                                                                       \
+        return cudaGetLastError();                                                           \
+    }
+    SD_SPREAD_LANES(4) SD_SPREAD_LANES(5) SD_SPREAD_LANES(6) SD_SPREAD_LANES(7) SD_SPREAD_LANES(8)
+#undef SD_SPREAD_LANES
 #define SD_SPREAD_CASE(WW)                                                                   \
     case WW: {                                                                               \
         auto kern = (dim == 2) ? k_spread<T, 2, WW> : k_spread<T, 3, WW>;                    \
@@ -1996,7 +2108,7 @@ cudaError_t launch_spread_x_t(const SpreadArgs<T>& a, const BinArgs& bn, int nbz
         if (a.m > 0) {
             k_bin_count_yz<float, 3, SX_W><<<gpts, 256, 0, st>>>(a, bn, SX_TY, SX_TZ);
             k_bin_scan<<<batch, 1024, 0, st>>>(bn);
-            k_bin_scatter<float><<<gpts, 256, 0, st>>>(a.m, bn);
+            k_records<<<dim3((unsigned)((a.m + 63) / 64), batch), 256, 0, st>>>(a, bn);
             note_launch(3);
         } else {
             k_bin_scan<<<batch, 1024, 0, st>>>(bn);
