@@ -707,12 +707,11 @@ static int prep_fields(sd_ctx* ctx, sd_shape* fx, const sd_grid* g, Prep** out, 
     CK(ctx, pool_alloc((void**)&F, Nd * sizeof(C), st));
     CK(ctx, pool_alloc((void**)&X, sx * sizeof(C), st));
     if (sy) CK(ctx, pool_alloc((void**)&Y, sy * sizeof(C), st));
-    CK(ctx, pool_alloc((void**)&Z, nd * sizeof(C), st));
+    CK(ctx, pool_alloc((void**)&Z, 2 * nd * sizeof(C), st));  // a pair of fields
     // type-2 tables on a grid of pitch n + w: the cells past n repeat the periodic field
     const int pn = n + ctx->p.w;
     const int64_t pd = (G.dim == 2) ? (int64_t)pn * pn : (int64_t)pn * pn * pn;
     CK(ctx, pool_alloc((void**)&Gf, 4 * pd * sizeof(C), st));
-    CK(ctx, cudaMemsetAsync(Gf, 0, 4 * pd * sizeof(C), st));
     for (int f = 0; f <= G.dim; ++f) {
         CK(ctx, launch_wtable<T>((const C*)p->B1, D, N, G.dim, G.L, ctx->p.sigma_g, 0, f - 1, F, st));
         RowArgs<T> r{};
@@ -741,7 +740,7 @@ static int prep_fields(sd_ctx* ctx, sd_shape* fx, const sd_grid* g, Prep** out, 
             c.out_outer_stride = (int64_t)n * n;
             CK(ctx, launch_cols<T>(COL_EXPAND, c, 1, st));
             c.in = Y;
-            c.out = Z;
+            c.out = Z + (f & 1) * nd;
             c.ncols = n * n;
             c.nouter = 1;
             c.in_outer_stride = 0;
@@ -749,12 +748,13 @@ static int prep_fields(sd_ctx* ctx, sd_shape* fx, const sd_grid* g, Prep** out, 
             CK(ctx, launch_cols<T>(COL_EXPAND, c, 1, st));
         } else {
             c.in = X;
-            c.out = Z;
+            c.out = Z + (f & 1) * nd;
             c.ncols = n;
             c.nouter = 1;
             CK(ctx, launch_cols<T>(COL_EXPAND, c, 1, st));
         }
-        CK(ctx, launch_interleave<T>(Z, Gf, n, pn, G.dim, f, st));
+        if ((f & 1) || f == G.dim)
+            CK(ctx, launch_interleave<T>(Z, (f & 1) ? Z + nd : nullptr, Gf, n, pn, G.dim, f >> 1, st));
     }
     pool_free(F, st);
     pool_free(X, st);
@@ -1839,8 +1839,11 @@ static int score_grad_t(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* movi
     a.beta = (T)ctx->p.beta;
     a.w = ctx->p.w;
     a.acc = (double*)acc;
+    a.score = (T*)score;
+    a.dq = (T*)dq;
+    a.dt = (T*)dt;
+    CK(ctx, cudaMemsetAsync(acc, 0, (size_t)P * 8 * sizeof(double), st));
     CK(ctx, launch_gather<T>(a, ctx->p.dim, st));
-    CK(ctx, launch_grad_finalize<T>((const double*)acc, (const T*)quats, P, ctx->p.dim, (T*)score, (T*)dq, (T*)dt, st));
     return SD_OK;
 }
 
@@ -1866,11 +1869,17 @@ static int refine_t(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* moving, 
     a.beta = (T)ctx->p.beta;
     a.w = ctx->p.w;
     a.acc = (double*)acc;
+    a.step = 1;
+    a.quats_io = (T*)quats;
+    a.trans_io = (T*)trans;
+    a.state = (double*)state;
+    a.rp = rp;
+    CK(ctx, cudaMemsetAsync(acc, 0, (size_t)P * 8 * sizeof(double), st));
     for (int k = 0; k <= steps; ++k) {
+        a.first = k == 0;
+        a.last = k == steps;
+        a.hist = hist ? (T*)hist + (int64_t)k * P : nullptr;
         CK(ctx, launch_gather<T>(a, ctx->p.dim, st));
-        T* h = hist ? (T*)hist + (int64_t)k * P : nullptr;
-        CK(ctx, launch_refine_step<T>((const double*)acc, (T*)quats, (T*)trans, (double*)state, P, ctx->p.dim, rp,
-                                      k == 0, h, k == steps, st));
     }
     return SD_OK;
 }

@@ -235,9 +235,10 @@ cudaError_t launch_reduce_topk(const double* part_score, const int* part_idx, in
 cudaError_t launch_reduce_argmax(const double* part_score, const int* part_idx, int nparts, int batch,
                                  int64_t rot0, void* cand, cudaStream_t st);
 
-// field f of 4 into its plane of the halo-padded type-2 tables
+// fields 2h and 2h + 1 of 4 into the halo-padded type-2 table (src1 null: zero)
 template <typename T>
-cudaError_t launch_interleave(const cplx<T>* src, cplx<T>* dst, int n, int pn, int dim, int f, cudaStream_t st);
+cudaError_t launch_interleave(const cplx<T>* src0, const cplx<T>* src1, cplx<T>* dst, int n, int pn, int dim, int h,
+                              cudaStream_t st);
 
 // ---- search -----------------------------------------------------------------
 // The k best of n candidates, best first; no scratch memory.
@@ -267,29 +268,36 @@ template <typename T>
 cudaError_t sort_by_morton(vec4<T>* pos, cplx<T>* c, int64_t m, double radius, int dim, cudaStream_t st);
 
 // ---- type-2 gather: score and gradient ---------------------------------------
+// Pose-update rule of the refinement loop (values of sd_refine_params.method).
+struct RefineParams {
+    int method;
+    double lr_t, lr_q, mass, inertia, damping, h;
+};
 template <typename T>
 struct GatherArgs {
     const vec4<T>* p2; const cplx<T>* c2; int64_t m2;
     const T* quats;           // P x 4
     const T* trans;           // P x 3
     int64_t P;
-    const cplx<T>* G;         // two planes of pn^d cells: (Phi, dPhi/dx), (dPhi/dy, dPhi/dz)
+    const cplx<T>* G;         // pn^d cells (Phi, dPhi/dx, dPhi/dy, dPhi/dz), 32-byte aligned
     int n;                    // periodic grid size per axis
-    int pn;                   // pitch of the planes: n plus a halo of w cells repeating the field
+    int pn;                   // pitch of the grid: n plus a halo of w cells repeating the field
     T inv_h, beta;
     int w;
-    double* acc;              // P x 8
+    double* acc;              // P x 8 (sums, CTAs done), zero before a launch and after it
+    int chunk;                // samples per CTA (set by launch_gather)
+    // what the last CTA of a pose does: write the gradient ...
+    T* score;                 // P
+    T* dq;                    // P x 4
+    T* dt;                    // P x 3
+    // ... or (step) update the pose in place
+    int step, first, last;    // first: no previous step's state; last: score only
+    T* quats_io;
+    T* trans_io;
+    T* hist;                  // P scores, or null
+    double* state;            // P x 12 (CG, dynamics)
+    RefineParams rp;
 };
 template <typename T> cudaError_t launch_gather(const GatherArgs<T>& a, int dim, cudaStream_t st);
-template <typename T> cudaError_t launch_grad_finalize(const double* acc, const T* quats, int64_t P, int dim,
-                                                       T* score, T* dq, T* dt, cudaStream_t st);
-// Pose-update rule of the refinement loop (values of sd_refine_params.method).
-struct RefineParams {
-    int method;
-    double lr_t, lr_q, mass, inertia, damping, h;
-};
-template <typename T> cudaError_t launch_refine_step(const double* acc, T* quats, T* trans, double* state, int64_t P,
-                                                     int dim, const RefineParams& rp, int first, T* hist, int last,
-                                                     cudaStream_t st);
 
 }  // namespace sd

@@ -2192,19 +2192,25 @@ __global__ void k_wtable(const cplx<T>* B1, const double* D, int N, int dim, dou
     W[i] = mk(T(vr), T(vi));
 }
 
-// Field f (0: Phi, 1-3: its gradient) of the type-2 tables into its plane:
-// plane f / 2 holds fields (2k, 2k + 1) of every cell side by side, on a grid of
-// pitch pn >= n per axis whose cells past n repeat the periodic field (a halo,
-// so that a tap box starting inside [0, n) never needs wrapping).
+// Two fields (h = 0: Phi and dPhi/dx, 1: dPhi/dy and dPhi/dz; src1 null: zero) into
+// the type-2 table, whose cells hold the four side by side, on a grid of pitch
+// pn >= n per axis whose cells past n repeat the periodic field (a halo, so that a
+// tap box starting inside [0, n) never needs wrapping).
 template <typename T>
-__global__ void k_interleave(const cplx<T>* src, cplx<T>* dst, int n, int pn, int dim, int f) {
+__global__ void k_interleave(const cplx<T>* src0, const cplx<T>* src1, cplx<T>* dst, int n, int pn, int dim, int h) {
     const int64_t cells = (dim == 3) ? (int64_t)pn * pn * pn : (int64_t)pn * pn;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= cells) return;
     const int x = (int)(i % pn), y = (int)((i / pn) % pn), z = (dim == 3) ? (int)(i / ((int64_t)pn * pn)) : 0;
     const int sx = x < n ? x : x - n, sy = y < n ? y : y - n, sz = z < n ? z : z - n;
     const int64_t si = (dim == 3) ? ((int64_t)sz * n + sy) * n + sx : (int64_t)sy * n + sx;
-    dst[(f >> 1) * 2 * cells + 2 * i + (f & 1)] = src[si];
+    const cplx<T> u = src0[si], v = src1 ? src1[si] : mk(T(0), T(0));
+    vec4<T> w;
+    w.x = u.x;
+    w.y = u.y;
+    w.z = v.x;
+    w.w = v.y;
+    reinterpret_cast<vec4<T>*>(dst)[2 * i + h] = w;
 }
 
 template <typename T>
@@ -2232,9 +2238,10 @@ cudaError_t launch_wshift_t(const cplx<T>* W, int N, int dim, int n, int s_h, cp
 }
 
 template <typename T>
-cudaError_t launch_interleave_t(const cplx<T>* src, cplx<T>* dst, int n, int pn, int dim, int f, cudaStream_t st) {
+cudaError_t launch_interleave_t(const cplx<T>* src0, const cplx<T>* src1, cplx<T>* dst, int n, int pn, int dim, int h,
+                                cudaStream_t st) {
     const int64_t cells = (dim == 3) ? (int64_t)pn * pn * pn : (int64_t)pn * pn;
-    k_interleave<T><<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(src, dst, n, pn, dim, f);
+    k_interleave<T><<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(src0, src1, dst, n, pn, dim, h);
     note_launch();
     return cudaGetLastError();
 }
@@ -2277,8 +2284,8 @@ cudaError_t launch_interleave_t(const cplx<T>* src, cplx<T>* dst, int n, int pn,
                                              cudaStream_t st) {                                                \
         return launch_wshift_t<T>(W, N, dim, n, s_h, out, st);                                          \
     }                                                                                                   \
-    template <> cudaError_t launch_interleave<T>(const cplx<T>* s, cplx<T>* d, int n, int pn, int dim, int f,       \
-                                                 cudaStream_t st) {                                                 \
-        return launch_interleave_t<T>(s, d, n, pn, dim, f, st);                                         \
+    template <> cudaError_t launch_interleave<T>(const cplx<T>* s0, const cplx<T>* s1, cplx<T>* d, int n, int pn,   \
+                                                 int dim, int h, cudaStream_t st) {                                 \
+        return launch_interleave_t<T>(s0, s1, d, n, pn, dim, h, st);                                    \
     }                                                                                                   \
     }
