@@ -550,11 +550,10 @@ def launch_count() -> int:
 
 
 def decode_cands(buf: torch.Tensor):
-    """(score float64, rot int32, idx int32) views of a candidate buffer."""
-    b = buf.reshape(-1, CAND_BYTES)
-    score = b[:, :8].contiguous().view(torch.float64).reshape(-1)
-    ri = b[:, 8:].contiguous().view(torch.int32).reshape(-1, 2)
-    return score, ri[:, 0], ri[:, 1]
+    """(score float64, rot int32, idx int32) of a candidate buffer (views of one copy of it)."""
+    b = buf.reshape(-1, CAND_BYTES).clone(memory_format=torch.contiguous_format)
+    ri = b.view(torch.int32)
+    return b.view(torch.float64)[:, 0], ri[:, 2], ri[:, 3]
 
 
 # ---------------------------------------------------------------------------
