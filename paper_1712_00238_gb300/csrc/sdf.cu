@@ -145,10 +145,15 @@ __device__ __forceinline__ void node_terms(T* v, const T d[3], const T N[3]) {
     v[23] = T(2) * (N[0] * yz + N[1] * xz + N[2] * xy);
 }
 
+// FP32 samples by twos for the paired instructions of the tree's direct sums: x0 x1
+// y0 y1 | z0 z1 Nx0 Nx1 | Ny0 Ny1 Nz0 Nz1, N = area times normal.  A pair past the end
+// repeats its last sample with N = 0.
+constexpr int PAIR = 12;
+
 template <typename T>
 __global__ void __launch_bounds__(SDF_TILE) k_sdf_nodes(const vec4<T>* bnd, const vec4<T>* nrm, int64_t n_b,
                                                         const float* tile_box, const float* sub_box, T* nodes,
-                                                        int64_t n_tiles) {
+                                                        int64_t n_tiles, float* pairs) {
     constexpr int NW = SDF_TILE / 32, NV = NODE - 4;
     __shared__ T part[NW][NV + 1];
     const int64_t i = (int64_t)blockIdx.x * SDF_TILE + threadIdx.x;
@@ -161,6 +166,14 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_nodes(const vec4<T>* bnd, cons
         nn = nrm[i];
     }
     const T N[3] = {nn.x * nn.w, nn.y * nn.w, nn.z * nn.w};
+    if constexpr (sizeof(T) == 4) {
+        if (i < (n_b + 1) / 2 * 2) {
+            const float4 pos = live ? q : bnd[n_b - 1];
+            float* w = pairs + (i >> 1) * PAIR + (i & 1);
+            w[0] = pos.x; w[2] = pos.y; w[4] = pos.z;
+            w[6] = N[0]; w[8] = N[1]; w[10] = N[2];
+        }
+    }
     for (int level = 0; level < 2; ++level) {
         const float* box = level ? sub_box + ((int64_t)blockIdx.x * NW + warp) * 6 : tile_box + (int64_t)blockIdx.x * 6;
         T c[3], d[3], v[NV], rho = T(0);
@@ -302,14 +315,18 @@ __device__ __forceinline__ bool node_far(const T* nd, const float lo[3], const f
 // Lanes test 32 tiles at a time; the warps share the far tiles, and each takes one
 // of a near tile's 8 sub-tiles, so they finish together.  Nodes and samples are
 // broadcast loads, four wavefronts per 16 bytes: the L1 data pipe is what bounds the
-// kernel (88 % at one query a lane), and two queries a lane halve them.
+// kernel (88 % at one query a lane), and two queries a lane halve them.  FP32 samples
+// are read and evaluated by twos (pairs) with paired instructions.  5,000 spheres
+// (199,433 queries, 320,000 samples): 3.0 ms, issuing on 70 % of cycles; the
+// cylinder (50,342, 20,000) 0.17 ms.
 constexpr int TREE_NW = 8;
 // Two queries a lane where that still gives every SM two CTAs.
 constexpr int64_t TREE_PAIR_MIN = 64 * 2 * 152;
 
 template <typename T, int Q>
-__global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T* nodes, const float* tile_box,
-                                                           const float* sub_box, int* list, int* list_n) {
+__global__ void __launch_bounds__(32 * TREE_NW, sizeof(T) == 4 ? 4 : 0) k_sdf_tree(SdfArgs<T> a, const T* nodes, const float* tile_box,
+                                                           const float* sub_box, const float* pairs, int* list,
+                                                           int* list_n) {
     constexpr int SUB = SDF_TILE / 32;
     static_assert(SUB == TREE_NW, "a tile's sub-tiles go to the warps");
     __shared__ T sh[3][TREE_NW][32 * Q];
@@ -348,8 +365,31 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T
     T dmin[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) dmin[q] = INFINITY;
+    float2 nx[Q], ny[Q], nz[Q];  // FP32: the negated points, doubled
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        nx[q] = make_float2(-(float)p[q].x, -(float)p[q].x);
+        ny[q] = make_float2(-(float)p[q].y, -(float)p[q].y);
+        nz[q] = make_float2(-(float)p[q].z, -(float)p[q].z);
+    }
     auto scan_sub = [&](int64_t j0) {  // the samples of one sub-tile
         const int cnt = (int)min((int64_t)32, a.n_b - j0);
+        if constexpr (sizeof(T) == 4) {
+            const float* b = pairs + (j0 >> 1) * PAIR;
+#pragma unroll 4
+            for (int k = 0; k < cnt; k += 2, b += PAIR) {
+                const float4 u = load4(b);
+                const float2 z = __ldg(reinterpret_cast<const float2*>(b + 4));
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    const float2 dx = __fadd2_rn(make_float2(u.x, u.y), nx[q]), dy = __fadd2_rn(make_float2(u.z, u.w), ny[q]),
+                                 dz = __fadd2_rn(z, nz[q]);
+                    const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+                    dmin[q] = fminf(dmin[q], fminf(d2.x, d2.y));
+                }
+            }
+            return;
+        }
         const vec4<T>* b = a.bnd + j0;
 #pragma unroll 4
         for (int k = 0; k < cnt; ++k) {
@@ -399,8 +439,12 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T
 
     // winding sum
     T wind[Q], err[Q], mag[Q];
+    float2 wind2[Q];
 #pragma unroll
-    for (int q = 0; q < Q; ++q) wind[q] = err[q] = mag[q] = T(0);
+    for (int q = 0; q < Q; ++q) {
+        wind[q] = err[q] = mag[q] = T(0);
+        wind2[q] = make_float2(0.f, 0.f);
+    }
     if (!a.pmc_override) {
         const T* subs = nodes + (int64_t)n_tiles * NODE;
         auto all_far = [&](const T* nd) {
@@ -441,6 +485,26 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T
                     node_eval<T, Q>(nd, p, wind, err, mag);
                     continue;
                 }
+                if constexpr (sizeof(T) == 4) {
+                    const float* b = pairs + (j0 >> 1) * PAIR;
+#pragma unroll 2
+                    for (int k = 0; k < cnt; k += 2, b += PAIR) {
+                        const float4 u = load4(b), v = load4(b + 4), w = load4(b + 8);
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) {
+                            const float2 dx = __fadd2_rn(make_float2(u.x, u.y), nx[q]),
+                                         dy = __fadd2_rn(make_float2(u.z, u.w), ny[q]),
+                                         dz = __fadd2_rn(make_float2(v.x, v.y), nz[q]);
+                            const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+                            const float2 r = make_float2(rsqrt_(d2.x), rsqrt_(d2.y));
+                            const float2 dot = __ffma2_rn(dz, make_float2(w.z, w.w),
+                                                          __ffma2_rn(dy, make_float2(w.x, w.y),
+                                                                     __fmul2_rn(dx, make_float2(v.z, v.w))));
+                            wind2[q] = __ffma2_rn(dot, __fmul2_rn(__fmul2_rn(r, r), r), wind2[q]);
+                        }
+                    }
+                    continue;
+                }
 #pragma unroll 4
                 for (int k = 0; k < cnt; ++k) {
                     const vec4<T> s = sample4(a.bnd + j0 + k), nn = sample4(a.nrm + j0 + k);
@@ -459,7 +523,7 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T
     constexpr double S = 4.0 * M_PI;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-        sh[1][warp][lane + 32 * q] = wind[q];
+        sh[1][warp][lane + 32 * q] = wind[q] + T(wind2[q].x + wind2[q].y);
         sh[2][warp][lane + 32 * q] = err[q] * T(G * 1.001f) + mag[q] * T(1e-4);
     }
     __syncthreads();
@@ -485,7 +549,7 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_tree(SdfArgs<T> a, const T
 
 // Membership of the listed queries from the sum over every sample.  Work items
 // (256 queries, a share of the tiles) are dealt to a fixed grid, so that a few
-// queries against many samples still fill it; the shares are added in order.
+// queries against many samples still fill it; a warp adds a query's shares.
 constexpr int LIST_CTAS = 152 * 8;
 __host__ __device__ __forceinline__ int list_splits(int chunks, int64_t n_tiles) {
     const int s = LIST_CTAS / (chunks > 0 ? chunks : 1);
@@ -530,10 +594,12 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_wind_list_finish(SdfArgs<T> a,
                                                                    const T* part) {
     const int n = *list_n, chunks = (n + SDF_TILE - 1) / SDF_TILE;
     const int splits = list_splits(chunks, a.n_tiles);
-    for (int e = blockIdx.x * SDF_TILE + (int)threadIdx.x; e < n; e += (int)gridDim.x * SDF_TILE) {
+    const int lane = threadIdx.x & 31;
+    for (int e = (blockIdx.x * SDF_TILE + (int)threadIdx.x) / 32; e < n; e += (int)gridDim.x * SDF_TILE / 32) {  // a warp each
         T wind = T(0);
-        for (int k = 0; k < splits; ++k) wind += part[(int64_t)k * chunks * SDF_TILE + e];
-        a.pmc[list[e]] = wind > T(2.0 * M_PI) ? int8_t(-1) : int8_t(1);
+        for (int k = lane; k < splits; k += 32) wind += part[(int64_t)k * chunks * SDF_TILE + e];
+        for (int off = 16; off > 0; off >>= 1) wind += __shfl_down_sync(0xffffffffu, wind, off);
+        if (lane == 0) a.pmc[list[e]] = wind > T(2.0 * M_PI) ? int8_t(-1) : int8_t(1);
     }
 }
 
@@ -884,26 +950,30 @@ static cudaError_t launch_nearest(const SdfArgs<T>& a, int dim, cudaStream_t st)
         const size_t nodes_bytes = (size_t)a.n_tiles * (1 + SDF_TILE / 32) * NODE * sizeof(T);
         const size_t parts = (size_t)SDF_TILE * (nb > LIST_CTAS ? nb : LIST_CTAS);
         const size_t list_bytes = ((size_t)a.m + 64) * sizeof(int) / 256 * 256 + 256;
-        if ((e = pool_alloc((void**)&scratch, nodes_bytes + list_bytes + parts * sizeof(T) + 256, st)) != cudaSuccess)
+        const size_t pairs_bytes = sizeof(T) == 4 ? (size_t)a.n_tiles * SDF_TILE / 2 * PAIR * sizeof(float) : 0;
+        if ((e = pool_alloc((void**)&scratch, nodes_bytes + list_bytes + parts * sizeof(T) + pairs_bytes + 512, st)) !=
+            cudaSuccess)
             return e;
         T* nodes = reinterpret_cast<T*>(scratch);
         int* list_n = reinterpret_cast<int*>(scratch + (nodes_bytes + 255) / 256 * 256);
         int* list = list_n + 1;
         T* part = reinterpret_cast<T*>(reinterpret_cast<char*>(list_n) + list_bytes);
+        float* pairs = reinterpret_cast<float*>(reinterpret_cast<char*>(part) + (parts * sizeof(T) + 255) / 256 * 256);
         e = cudaMemsetAsync(list_n, 0, sizeof(int), st);
         if (e != cudaSuccess) {
             pool_free(scratch, st);
             return e;
         }
         const float* sub_box = a.tree_box + a.n_tiles * 6;
-        if (!a.pmc_override) {
-            k_sdf_nodes<T><<<(unsigned)a.n_tiles, SDF_TILE, 0, st>>>(a.bnd, a.nrm, a.n_b, a.tree_box, sub_box, nodes, a.n_tiles);
-            note_launch();
-        }
+        k_sdf_nodes<T><<<(unsigned)a.n_tiles, SDF_TILE, 0, st>>>(a.bnd, a.nrm, a.n_b, a.tree_box, sub_box, nodes,
+                                                                 a.n_tiles, pairs);
+        note_launch();
         if (sizeof(T) == 4 && a.m >= TREE_PAIR_MIN)
-            k_sdf_tree<T, 2><<<(unsigned)((a.m + 63) / 64), 32 * TREE_NW, 0, st>>>(a, nodes, a.tree_box, sub_box, list, list_n);
+            k_sdf_tree<T, 2><<<(unsigned)((a.m + 63) / 64), 32 * TREE_NW, 0, st>>>(a, nodes, a.tree_box, sub_box, pairs, list,
+                                                                                         list_n);
         else
-            k_sdf_tree<T, 1><<<(unsigned)((a.m + 31) / 32), 32 * TREE_NW, 0, st>>>(a, nodes, a.tree_box, sub_box, list, list_n);
+            k_sdf_tree<T, 1><<<(unsigned)((a.m + 31) / 32), 32 * TREE_NW, 0, st>>>(a, nodes, a.tree_box, sub_box, pairs, list,
+                                                                                         list_n);
         note_launch();
         if (!a.pmc_override) {
             k_sdf_wind_list<T><<<LIST_CTAS, SDF_TILE, 0, st>>>(a, list, list_n, part);
