@@ -108,10 +108,12 @@ struct TwStage {
 
 // Steps a pass runs inside its transform, once in every thread: loaded() after the
 // first stage's loads are issued (what it writes to shared memory is visible from
-// the second stage on), drained() after the barrier that ends the last stage's
-// reads of the line buffer, before its butterflies.
+// the second stage on), staged() after the barrier that ends the first of several
+// stages (every thread has its inputs), drained() after the barrier that ends the last
+// stage's reads of the line buffer, before its butterflies.
 struct NoHook {
     __device__ __forceinline__ void loaded() const {}
+    __device__ __forceinline__ void staged() const {}
     __device__ __forceinline__ void drained() const {}
 };
 template <typename F>
@@ -121,12 +123,20 @@ struct LoadedHook : NoHook {
     __device__ __forceinline__ void loaded() const { f(); }
 };
 template <typename F, typename G>
-struct Hooks {
+struct Hooks : NoHook {
     F f;
     G g;
     __device__ __forceinline__ Hooks(F a, G b) : f(a), g(b) {}
     __device__ __forceinline__ void loaded() const { f(); }
     __device__ __forceinline__ void drained() const { g(); }
+};
+template <typename F, typename G>
+struct StagedHooks : NoHook {
+    F f;
+    G g;
+    __device__ __forceinline__ StagedHooks(F a, G b) : f(a), g(b) {}
+    __device__ __forceinline__ void loaded() const { f(); }
+    __device__ __forceinline__ void staged() const { g(); }
 };
 
 // Line transforms of NL lines per block of NT threads (see fft_lines_io for the
@@ -203,6 +213,7 @@ __device__ __forceinline__ void fftp_lines(C* buf, int ld, const C* tw, Load& lo
     }
     if constexpr (!last) {
         __syncthreads();
+        if constexpr (first) hook.staged();
         fftp_lines<C, LEN, INV, NL, NT, LAY, PAD, SRC_SMEM, HALF_IN, S + 1, P * R>(buf, ld, tw, load, emit, hook);
     }
 }

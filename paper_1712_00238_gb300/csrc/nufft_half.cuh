@@ -240,8 +240,15 @@ __global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_inv_min_ctas<T, LE
     fftp_lines<C, LEN, true, TC, NT, LAY_COL, false, false, false>(buf, LD, a.twI, load, emit);
 }
 
-// CTAs per SM a row pass leaves before its CTAs take more groups (12 to 48 measure alike).
-constexpr int HALF_ROW_WAVE = 24;
+// A row pass leaves this many CTAs per SM before its CTAs take more groups, up to a
+// most each: the copies then run ahead, and a K-best merge (K block-wide rounds) is
+// paid once.  68 rotations at N = 128: 161 us without bulk copies, 148 with; 60 at
+// N = 192: 521 -> 461 (with one comparison per butterfly where each output took one);
+// 77 at N = 96 keeping four: 174 -> 133 (8 CTAs per SM, 32 groups; 160 at 16 and 16).
+template <int K>
+__host__ __device__ constexpr int half_row_wave() { return K == 1 ? 16 : 8; }
+template <int K>
+__host__ __device__ constexpr int half_row_most() { return K == 1 ? 16 : 32; }
 // Register bound of the row pass: the two rows' running best take it past the 40
 // registers of six CTAs (192 points spilled: 247 us per 20 rotations against 175 at four).
 template <int K>
@@ -249,6 +256,44 @@ __host__ __device__ constexpr int rows_half_min_ctas() { return K == 1 ? 4 : (K 
 
 // Inverse x of packed lines.  Row groups of TR lines (2 TR rows) are handled by one
 // CTA in turn: its K best are kept in registers across the groups and merged once.
+// Whether a row pass's groups come in by bulk copies (two-stage FP32 lines; an FP64
+// CTA's raw lines would cost it its shared memory).
+template <typename T, int LEN>
+__host__ __device__ constexpr bool rows_half_bulk() {
+    return sizeof(T) == 4 && plan_radix(LEN, 1) != 0;
+}
+template <typename T, int LEN, int K>
+__host__ __device__ constexpr size_t rows_half_smem() {
+    constexpr int TR = lines_per_cta<T, LEN>(), NT = cta_threads<T, LEN>();
+    return (size_t)(TR * ((rows_half_bulk<T, LEN>() ? LEN : 0) + line_pitch(LEN)) + tw_count(LEN)) * sizeof(cplx<T>) +
+           (K > 1 ? (size_t)NT * K * (sizeof(T) + sizeof(int)) : 0);
+}
+
+// One bulk copy (bytes and both addresses multiples of 16) that reports to an
+// mbarrier, and the bounded wait for its phase.
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst), b = (unsigned)__cvta_generic_to_shared(bar);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d), "l"(src),
+                 "r"(bytes), "r"(b)
+                 : "memory");
+}
+__device__ __forceinline__ bool bulk_wait(uint64_t* bar, unsigned phase) {
+    const unsigned b = (unsigned)__cvta_generic_to_shared(bar);
+    for (int tries = 0; tries < (1 << 22); ++tries) {
+        unsigned ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok)
+                     : "r"(b), "r"(phase)
+                     : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
+__device__ __forceinline__ float max_num(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_num(double a, double b) { return a > b || b != b ? a : b; }  // as fmax, but cheap
+
 template <typename T, int LEN, int K>
 __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
     using C = cplx<T>;
@@ -257,50 +302,102 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
     constexpr int LD = line_pitch(LEN);
     constexpr int NTW = tw_count(LEN);
     constexpr int NB1 = LEN / plan_radix(LEN, 0);
-    constexpr int PL = LEN / plan_last_radix(LEN);
-    constexpr bool one_bfly = TR * (LEN / plan_last_radix(LEN)) <= NT;
+    constexpr int RL = plan_last_radix(LEN), PL = LEN / RL;
+    constexpr bool BULK = rows_half_bulk<T, LEN>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* buf = reinterpret_cast<C*>(smem_raw);
+    C* raw = reinterpret_cast<C*>(smem_raw);
+    C* buf = raw + (BULK ? TR * LEN : 0);
     C* tw = buf + TR * LD;
-    TwStage<C, NTW, NT> tws;
-    tws.load(a.tw);
     constexpr int NH = LEN / 2;
     const C* in = a.in + (int64_t)blockIdx.y * a.in_rot_stride;
     const int nlines = a.nrows / 2, ngroups = (nlines + TR - 1) / TR;
+    // a group's lines are contiguous: one bulk copy brings the next group in while this
+    // one is in its second stage
+    __shared__ __align__(8) uint64_t bar;
+    auto fetch = [&](int g) {
+        if (g < ngroups)
+            bulk_copy(raw, in + (int64_t)g * TR * LEN, (unsigned)(min(TR, nlines - g * TR) * LEN * sizeof(C)), &bar);
+    };
+    if constexpr (BULK) {
+        if (threadIdx.x == 0) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&bar)) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            fetch(blockIdx.x);
+        }
+        __syncthreads();
+    }
+    unsigned phase = 0;
+    bool lost = false;
+    TwStage<C, NTW, NT> tws;
+    tws.load(a.tw);
     const C zero = mk(T(0), T(0));
     T bestA = -INFINITY, bestB = -INFINITY;
     int idxA = INT_MAX, idxB = INT_MAX;
     TopK<T, K> top;
     if constexpr (K > 1) top.init();
+    C keep[RL];
     for (int g = blockIdx.x; g < ngroups; g += gridDim.x) {
         const int line0 = g * TR;
         const int nl = nlines - line0;
         const C* src = in + (int64_t)line0 * LEN;
+        if constexpr (BULK) {
+            lost |= !bulk_wait(&bar, phase);  // (a copy that never came: the CTA finds nothing)
+            phase ^= 1;
+        }
         auto load = [&](int line, int i, int r) -> C {
-            return line < nl ? src[line * LEN + i + r * NB1] : zero;
+            return line < nl ? (BULK ? raw : src)[line * LEN + i + r * NB1] : zero;
         };
+        // a butterfly's outputs are kept until all are there: one maximum each, and the
+        // comparisons with what the thread holds only where that maximum could enter it
         auto emit = [&](int line, int i, int r, C v) {
-            if (line >= nl) return;
+            keep[r] = v;
+            if (r < RL - 1 || line >= nl) return;
+            T mA = keep[0].x, mB = keep[0].y;
+#pragma unroll
+            for (int q = 1; q < RL; ++q) {
+                mA = max_num(mA, keep[q].x);
+                mB = max_num(mB, keep[q].y);
+            }
             // line (z, y), y < N/2, holds rows (z, y) and (z, y + N/2)
-            const int l = line0 + line, o = (l + l / NH * NH) * LEN + i + r * PL;
+            const int l = line0 + line, o = (l + l / NH * NH) * LEN + i;
             if constexpr (K > 1) {
-                top.push(v.x, o);
-                top.push(v.y, o + NH * LEN);
-            } else if constexpr (one_bfly) {
-                // outputs (and groups) come in increasing index order: a strict
-                // comparison keeps the lowest index of equal values
-                if (v.x > bestA) { bestA = v.x; idxA = o; }
-                if (v.y > bestB) { bestB = v.y; idxB = o + NH * LEN; }
+                if (mA >= top.v[K - 1])
+#pragma unroll
+                    for (int q = 0; q < RL; ++q) top.push(keep[q].x, o + q * PL);
+                if (mB >= top.v[K - 1])
+#pragma unroll
+                    for (int q = 0; q < RL; ++q) top.push(keep[q].y, o + NH * LEN + q * PL);
             } else {
-                argmax_merge(bestA, idxA, v.x, o);
-                argmax_merge(bestB, idxB, v.y, o + NH * LEN);
+                // a thread's outputs (and groups) come in increasing index order: strict
+                // comparisons keep the lowest index of equal values
+                if (mA > bestA) {
+#pragma unroll
+                    for (int q = 0; q < RL; ++q)
+                        if (keep[q].x > bestA) { bestA = keep[q].x; idxA = o + q * PL; }
+                }
+                if (mB > bestB) {
+#pragma unroll
+                    for (int q = 0; q < RL; ++q)
+                        if (keep[q].y > bestB) { bestB = keep[q].y; idxB = o + NH * LEN + q * PL; }
+                }
             }
         };
-        fftp_lines<C, LEN, true, TR, NT, LAY_ROW, true, false, false>(buf, LD, tw, load, emit, LoadedHook([&] {
-            if (g == (int)blockIdx.x) tws.store(tw);
-        }));
+        fftp_lines<C, LEN, true, TR, NT, LAY_ROW, true, false, false>(
+            buf, LD, tw, load, emit,
+            StagedHooks(
+                [&] {
+                    if (g == (int)blockIdx.x) tws.store(tw);
+                },
+                [&] {
+                    if (BULK && threadIdx.x == 0) fetch(g + gridDim.x);
+                }));
         // the next group's first writes to buf come after the barrier that follows
         // this group's last reads
+    }
+    if (BULK && lost) {
+        bestA = bestB = -INFINITY;
+        idxA = idxB = INT_MAX;
+        if constexpr (K > 1) top.init();
     }
     if constexpr (K > 1) {
         T* sv = reinterpret_cast<T*>(tw + NTW);
@@ -450,15 +547,12 @@ static cudaError_t rows_half_launch(const RowArgs<T>& a, int batch, int* nparts,
     const int ngroups = (a.nrows / 2 + TR - 1) / TR;
     if (nparts) *nparts = 0;
     if (ngroups == 0 || batch == 0) return cudaSuccess;
-    // groups per CTA: enough to amortise its merge, few enough to leave several
-    // waves of CTAs (the K-best merge costs about as much as a group's transform)
     const int64_t total = (int64_t)ngroups * batch;
-    int G = (int)(total / (HALF_ROW_WAVE * 152));
-    G = G < 1 ? 1 : (G > 8 ? 8 : G);
+    int G = (int)(total / (half_row_wave<K>() * 152));
+    G = G < 1 ? 1 : (G > half_row_most<K>() ? half_row_most<K>() : G);
     const int nb = (ngroups + G - 1) / G;
     if (nparts) *nparts = nb * K;
-    const size_t smem = (size_t)(TR * line_pitch(LEN) + tw_count(LEN)) * sizeof(cplx<T>) +
-                        (K > 1 ? (size_t)NT * K * (sizeof(T) + sizeof(int)) : 0);
+    constexpr size_t smem = rows_half_smem<T, LEN, K>();
     auto kern = k_rows_half<T, LEN, K>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
