@@ -1,4 +1,4 @@
-// Batched line FFTs in shared memory: mixed radix (2, 3, 4, 8, 12, 16, 24) Stockham
+// Batched line FFTs in shared memory: mixed radix (2, 3, 4, 8, 12, 16, 24, 32) Stockham
 // autosort stages (Van Loan, "Computational Frameworks for the FFT", 1992).
 //
 // Each stage of radix R over a line of LEN points takes, for every butterfly
@@ -36,7 +36,7 @@ __host__ __device__ constexpr int plan_radix(int len, int s) {
         case 192: return s == 0 ? 16 : (s == 1 ? 12 : 0);
         case 256: return s == 0 ? 16 : (s == 1 ? 16 : 0);
         case 384: return s == 0 ? 24 : (s == 1 ? 16 : 0);
-        case 512: return s == 0 ? 8 : (s == 1 ? 8 : (s == 2 ? 8 : 0));
+        case 512: return s == 0 ? 32 : (s == 1 ? 16 : 0);
         default: return 0;
     }
 }
@@ -101,6 +101,36 @@ __host__ __device__ __forceinline__ C w24(int m) {
     }
     T x, y;  // exp(-i theta) rotated by (-i)^quadrant
     switch ((m / 6) & 3) {
+        case 0: x = c; y = -s; break;
+        case 1: x = -s; y = -c; break;
+        case 2: x = -c; y = s; break;
+        default: x = s; y = c; break;
+    }
+    return INV ? mk(x, -y) : mk(x, y);
+}
+
+// exp(-+2 pi i m / 32), m in [0, 32): sixteenths of pi as constants, cos(k pi / 16) for
+// k = 0..8, reflected and rotated by quadrant.
+template <bool INV, typename C>
+__host__ __device__ __forceinline__ C w32(int m) {
+    using T = decltype(C{}.x);
+    auto cosk = [](int k) -> T {  // k in [0, 8]
+        switch (k) {
+            case 0: return T(1);
+            case 1: return T(0.98078528040323044913);
+            case 2: return T(0.92387953251128675613);
+            case 3: return T(0.83146961230254523708);
+            case 4: return T(0.70710678118654752440);
+            case 5: return T(0.55557023301960222474);
+            case 6: return T(0.38268343236508977173);
+            case 7: return T(0.19509032201612826785);
+            default: return T(0);
+        }
+    };
+    const int k = m % 8;
+    const T c = cosk(k), s = cosk(8 - k);  // cos and sin of k pi / 16
+    T x, y;                                // exp(-i theta) rotated by (-i)^quadrant
+    switch ((m / 8) & 3) {
         case 0: x = c; y = -s; break;
         case 1: x = -s; y = -c; break;
         case 2: x = -c; y = s; break;
@@ -183,6 +213,24 @@ __host__ __device__ __forceinline__ void dft(C* v) {
             C x0 = b[0][k1], x1 = b[1][k1], x2 = b[2][k1], x3 = b[3][k1];
             dft4<INV>(x0, x1, x2, x3);
             v[k1] = x0; v[k1 + 4] = x1; v[k1 + 8] = x2; v[k1 + 12] = x3;
+        }
+    } else if constexpr (R == 32) {
+        // n = 8 n1 + n2, k = k1 + 4 k2
+        C b[4][8];
+#pragma unroll
+        for (int n2 = 0; n2 < 8; ++n2) {
+            C t0 = v[n2], t1 = v[8 + n2], t2 = v[16 + n2], t3 = v[24 + n2];
+            dft4<INV>(t0, t1, t2, t3);
+            b[0][n2] = t0;
+            b[1][n2] = n2 == 0 ? t1 : cmul(t1, w32<INV, C>(n2));
+            b[2][n2] = n2 == 0 ? t2 : cmul(t2, w32<INV, C>(2 * n2));
+            b[3][n2] = n2 == 0 ? t3 : cmul(t3, w32<INV, C>(3 * n2));
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+            dft<8, INV>(b[k1]);
+#pragma unroll
+            for (int k2 = 0; k2 < 8; ++k2) v[k1 + 4 * k2] = b[k1][k2];
         }
     } else if constexpr (R == 12) {
         dft3q<4, INV>(v);

@@ -57,6 +57,27 @@ __device__ __forceinline__ void dft_lowhalf(C* v) {
             dft4<INV>(x0, x1, x2, x3);
             v[k1] = x0; v[k1 + 4] = x1; v[k1 + 8] = x2; v[k1 + 12] = x3;
         }
+    } else if constexpr (R == 32) {
+        // n = 8 n1 + n2, k = k1 + 4 k2; the 4-point DFTs see (a0, a1, 0, 0)
+        C b[4][8];
+#pragma unroll
+        for (int n2 = 0; n2 < 8; ++n2) {
+            const C a0 = v[n2], a1 = v[8 + n2];
+            b[0][n2] = cadd(a0, a1);
+            b[1][n2] = add_mi<INV>(a0, a1);
+            b[2][n2] = csub(a0, a1);
+            b[3][n2] = sub_mi<INV>(a0, a1);
+        }
+#pragma unroll
+        for (int n2 = 1; n2 < 8; ++n2)
+#pragma unroll
+            for (int k1 = 1; k1 < 4; ++k1) b[k1][n2] = cmul(b[k1][n2], w32<INV, C>(n2 * k1));
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+            dft<8, INV>(b[k1]);
+#pragma unroll
+            for (int k2 = 0; k2 < 8; ++k2) v[k1 + 4 * k2] = b[k1][k2];
+        }
     } else if constexpr (R == 8) {
         // even / odd inputs each (a0, a1, 0, 0)
         const T r = T(0.70710678118654752440);

@@ -28,11 +28,15 @@ namespace sd {
 // the other way, 68 rotations at N = 128: 562 against 524).
 template <int LENF>
 __host__ __device__ constexpr bool half_tw_smem() { return LENF <= 256; }
-// The asynchronous copies of the mirror column and the table (see the body) hide two
-// global latencies a CTA: 652 -> 562 us at 256 points, 1354 -> 1171 at 512.  384 points
-// are issue- and register-bound (56 a thread): 1914 us without, 2081 with them.
+// Asynchronous copies of the table (W) and of the mirror column (B, see the body) hide
+// a global latency each, but take registers and address arithmetic.  Fused pass, us, with
+// neither / B only / W only / both: 192 points (64 rotations, N = 96) - / 256 / 271 / 255;
+// 256 points (68, N = 128) 652 / - / 552 / 568; 384 points (60, N = 192) 1904 / 2003 /
+// 1992 / 2081; 512 points (12, N = 256) - / 948 / - / 995.
 template <int LENF>
-__host__ __device__ constexpr bool half_prefetch() { return LENF != 384; }
+__host__ __device__ constexpr bool half_prefetch_w() { return LENF <= 256; }
+template <int LENF>
+__host__ __device__ constexpr bool half_prefetch_b() { return LENF != 256 && LENF != 384; }
 
 template <typename T, int LENF, int TC>
 __host__ __device__ constexpr size_t cols_half_smem() {
@@ -127,7 +131,7 @@ __device__ __forceinline__ void cols_half_body(const ColArgs<T>& a) {
             return o < LENI / 2 ? o : (o >= LENF - LENI / 2 ? o - LENI : -1);
         }
     };
-    constexpr bool PF = half_prefetch<LENF>();
+    constexpr bool PFW = half_prefetch_w<LENF>(), PFB = half_prefetch_b<LENF>();
     constexpr int R1 = plan_radix(LENF, 0), RL = plan_last_radix(LENF), RIN = PRUNED ? R1 / 2 : R1;
     const int line = (int)threadIdx.x % TC;
     const C *twF = a.twF, *twI = a.twI;
@@ -159,7 +163,6 @@ __device__ __forceinline__ void cols_half_body(const ColArgs<T>& a) {
         copy_commit();
     };
     auto fetchB = [&] {
-        copy_wait();  // the table's copies
 #pragma unroll
         for (int q = 0; q < (TC * NB1 + NT - 1) / NT; ++q) {
             const int t = threadIdx.x + q * NT;
@@ -176,12 +179,12 @@ __device__ __forceinline__ void cols_half_body(const ColArgs<T>& a) {
         const int kp = slot(i, r);
         if (kp >= 0 && ok) {
             C* g = acc + line * LDA + kp;
-            *g = cmul(v, PF ? *g : WA[kp * hcols]);
+            *g = cmul(v, PFW ? *g : WA[kp * hcols]);
         }
     };
     auto loadB = [&](int, int i, int r) -> C {
         const int e = cell(i, r);
-        if (PF) return (ok && e < s) ? cconj(buf[e * TC + line]) : zero;
+        if (PFB) return (ok && e < s) ? cconj(buf[e * TC + line]) : zero;
         return (ok && e < s) ? cconj(inB[e * ncols]) : zero;
     };
     auto emitB = [&](int, int i, int r, C v) {  // the entries this thread wrote in emitA
@@ -191,17 +194,20 @@ __device__ __forceinline__ void cols_half_body(const ColArgs<T>& a) {
             *g = cadd(*g, cmul(v, WB[kp * hcols]));
         }
     };
-    if constexpr (PF) {
-        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadA, emitA,
-                                                                          Hooks(fetchW, fetchB));
-        copy_wait();
-        // the barrier of loaded(): every thread has read its cells before buf is rewritten
-        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadB, emitB,
-                                                                          LoadedHook([] { __syncthreads(); }));
-    } else {
-        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadA, emitA);
-        fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadB, emitB);
-    }
+    fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadA, emitA,
+                                                                      Hooks(
+                                                                          [&] {
+                                                                              if constexpr (PFW) fetchW();
+                                                                          },
+                                                                          [&] {
+                                                                              if constexpr (PFW) copy_wait();
+                                                                              if constexpr (PFB) fetchB();
+                                                                          }));
+    if constexpr (PFB) copy_wait();
+    // with copies, the barrier of loaded(): every thread has read its cells before buf is rewritten
+    fftp_lines<C, LENF, false, TC, NT, LAY_COL, false, false, PRUNED>(buf, LD, twF, loadB, emitB, LoadedHook([] {
+                                                                          if constexpr (PFB) __syncthreads();
+                                                                      }));
     __syncthreads();
     if constexpr (PACK) {
         PackEmit<C, LENI> emit_out{out, kx, ok};

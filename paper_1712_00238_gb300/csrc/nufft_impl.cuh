@@ -45,9 +45,9 @@ __host__ __device__ constexpr int lines_per_cta() {
 
 // Threads of a line-pass CTA: the butterflies of the plan's widest stage over
 // the CTA's lines (one butterfly per thread per stage), rounded up to whole
-// warps, at least 64.  Wider than 384 butterflies (512-point lines) the CTA
-// keeps 256 threads with two butterflies each: registers would otherwise allow
-// only one CTA per SM.
+// warps, at least 64.  Wider than 384 butterflies (the radix-16 stage of 512-point
+// lines) the CTA keeps 256 threads with two butterflies each: registers would
+// otherwise allow only one CTA per SM.
 template <int LEN>
 __host__ __device__ constexpr int cta_threads_for(int lines) {
     int most = 0;
@@ -67,7 +67,7 @@ __host__ __device__ constexpr int cta_threads() {
 // Resident CTAs per SM that a pass's register allocation is bounded for, 0 for
 // the compiler's own choice.  The 384-point FP32 passes (384 threads) take 3
 // (at most 56 registers a thread; 66-70 otherwise, which allows two); the
-// 512-point FP32 passes take 2 (at most 128; 150-170 otherwise, one CTA); the
+// 512-point FP32 passes (256 threads, radix 32 first) take 2 (at most 128); the
 // fused 256-point column pass takes 4 (at most 64; it would take 75).  Every
 // other pass keeps the compiler's choice, which already allows four or more
 // CTAs of 256 threads: an explicit minimum there makes it take more registers
@@ -1646,8 +1646,8 @@ __global__ void __cluster_dims__(IYX_CS, 1, 1) __launch_bounds__(iyx_threads<T, 
 }
 
 // Resident CTAs per SM the pruned passes are compiled for (0: the compiler's choice).
-// 512-point FP32 lines (256 threads, two butterflies each) take 2 (at most 128
-// registers; 146 otherwise); 384-point ones 3 (384 threads: at most 56).
+// 512-point FP32 lines (256 threads, radix 32 first) take 2 (at most 128 registers);
+// 384-point ones 3 (384 threads: at most 56).
 template <typename T, int LEN, int KIND>
 __host__ __device__ constexpr int pruned_min_ctas() {
     return sizeof(T) != 4 ? 0 : (LEN == 512 ? 2 : (LEN == 384 ? 3 : 0));
