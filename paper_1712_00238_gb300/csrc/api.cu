@@ -580,7 +580,7 @@ static int spread_x_bins(int s, int* nby, int* nbz) {
 static size_t bins_bytes_x(int s, int64_t m, int batch) {
     int nby, nbz;
     const int nbins = spread_x_bins(s, &nby, &nbz);
-    return (((size_t)batch * (3 * (size_t)nbins + 1) + 3 * (size_t)batch * (size_t)m + 3) / 4 * 4 +
+    return (((size_t)batch * ((3 + SPREADX_XC) * (size_t)nbins + 1) + 3 * (size_t)batch * (size_t)m + 3) / 4 * 4 +
             (size_t)batch * (size_t)m * SPREADX_REC) * sizeof(int);
 }
 static void bins_layout_x(void* p, int s, int64_t m, int batch, BinArgs* bn, int* nbz) {
@@ -594,6 +594,8 @@ static void bins_layout_x(void* p, int s, int64_t m, int batch, BinArgs* bn, int
     q += (size_t)batch * nbins;
     bn->cmax = q;
     q += (size_t)batch * nbins;
+    bn->xcount = q;
+    q += (size_t)batch * nbins * SPREADX_XC;
     bn->offset = q;
     q += (size_t)batch * (nbins + 1);
     bn->bin_of = q;
@@ -827,10 +829,15 @@ struct Search {
     int nbz = 0;  // SPREAD_X: bins along z
 };
 
+// A batch's records of fused spreading (108 bytes a sample and rotation with the bins)
+// stay below 7 GB; larger jobs spread directly.
+template <typename T>
+static bool spread_x_fits(const Search<T>& S, int batch) { return S.moving->m * batch <= (int64_t)1 << 26; }
+
 // Spreading fused with the x transform: pruned 3D FP32 searches with w = 6.
 template <typename T>
-static bool spread_x_ok(const sd_ctx* ctx, const Search<T>& S) {
-    return sizeof(T) == 4 && S.G.dim == 3 && ctx->p.w == 6 && S.plan.fft != SD_FFT_FULL;
+static bool spread_x_ok(const sd_ctx* ctx, const Search<T>& S, int batch) {
+    return sizeof(T) == 4 && S.G.dim == 3 && ctx->p.w == 6 && S.plan.fft != SD_FFT_FULL && spread_x_fits(S, batch);
 }
 
 // The forward-pass plans a job can run: FULL always, the pruned ones where the
@@ -876,7 +883,7 @@ static int search_setup(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* movi
     S->plan.fft = fft_plan_default(ctx, *S);
     S->iyx = ctx->opt_inv_cluster && sizeof(T) == 4 && S->G.dim == 3 && inv_yx_supported(S->G.N);
     if (ctx->opt_spread_box && bins_supported(ctx)) S->plan.bins = SPREAD_BOX;
-    if (ctx->opt_spread_fused && spread_x_ok(ctx, *S)) S->plan.bins = SPREAD_X;
+    if (ctx->opt_spread_fused && spread_x_ok(ctx, *S, S->plan.B)) S->plan.bins = SPREAD_X;
     return SD_OK;
 }
 
@@ -1071,7 +1078,7 @@ static int autotune(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
     auto it = ctx->tuned.find(key);
     if (it != ctx->tuned.end()) {
         S->plan.B = (int)std::min<int64_t>(it->second.B, std::max<int64_t>(S->n_r, 1));
-        S->plan.bins = it->second.bins;
+        if (it->second.bins != SPREAD_X || spread_x_fits(*S, S->plan.B)) S->plan.bins = it->second.bins;
         if (ctx->opt_fft_plan < 0 && fft_plan_ok(*S, it->second.fft)) S->plan.fft = it->second.fft;
         return SD_OK;
     }
@@ -1082,7 +1089,7 @@ static int autotune(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
     for (int B : {b0 / 4, b0 / 2, b0, 2 * b0}) {
         if (B < 1 || B > 64 || (B > S->n_r && B != b0)) continue;
         for (int bins : {0, SPREAD_BOX, SPREAD_X, 8, 12, 16}) {
-            if (bins == SPREAD_X ? !spread_x_ok(ctx, *S) : (bins && !bins_supported(ctx))) continue;
+            if (bins == SPREAD_X ? !spread_x_ok(ctx, *S, B) : (bins && !bins_supported(ctx))) continue;
             bool dup = false;
             for (auto& c : cand) dup |= (c.B == B && c.bins == bins);
             if (!dup) cand.push_back(Plan{B, bins, f0});
@@ -1706,12 +1713,12 @@ int sd_search_plan(sd_ctx* ctx, const sd_shape* moving, const sd_grid* g, int64_
         S.alt_cols = S.prunable && sizeof(T) == 4 && S.G.n >= 128 && S.G.n <= 384;
         S.plan.fft = fft_plan_default(ctx, S);
         if (ctx->opt_spread_box && bins_supported(ctx)) S.plan.bins = SPREAD_BOX;
-        if (ctx->opt_spread_fused && spread_x_ok(ctx, S)) S.plan.bins = SPREAD_X;
+        if (ctx->opt_spread_fused && spread_x_ok(ctx, S, S.plan.B)) S.plan.bins = SPREAD_X;
         if (ctx->opt_autotune && !ctx->opt_plain && ctx->opt_batch <= 0) {
             auto it = ctx->tuned.find(plan_key(ctx, S));
             if (it != ctx->tuned.end()) {
                 S.plan.B = (int)std::min<int64_t>(it->second.B, n_r);
-                S.plan.bins = it->second.bins;
+                if (it->second.bins != SPREAD_X || spread_x_fits(S, S.plan.B)) S.plan.bins = it->second.bins;
                 if (ctx->opt_fft_plan < 0 && fft_plan_ok(S, it->second.fft)) S.plan.fft = it->second.fft;
             }
         }

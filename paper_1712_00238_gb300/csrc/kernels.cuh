@@ -92,6 +92,7 @@ struct BinArgs {
     int* rank;            // batch x m
     int32_t* sorted;      // batch x m: sample indices in bin order
     int32_t* org;         // batch x m: packed tap-box origin (x | y << 10 | z << 20), fused spreading only
+    int* xcount;          // batch x nbins x SPREADX_XC, right after cmax: samples per 32 cells of x, fused spreading only
     float* rec;           // batch x m x SPREADX_REC: records in bin order, fused spreading only (no `sorted`)
 };
 // Spread by bins; accumulates into the batch's sub-boxes, which must be cleared first.
@@ -112,7 +113,7 @@ template <typename T> cudaError_t launch_spread_box(const SpreadArgs<T>& a, int 
 // sides are at least w - 1, so a tap box meets at most 2 x 2 bins; 6 x 6 rows
 // keep a CTA's shared memory to three CTAs per SM at n = 384 (measured faster
 // than 5 x 6).
-constexpr int SPREADX_TY = 6, SPREADX_TZ = 6, SPREADX_REC = 24;
+constexpr int SPREADX_TY = 6, SPREADX_TZ = 6, SPREADX_REC = 24, SPREADX_XC = 8;
 template <typename T>
 cudaError_t launch_spread_x(const SpreadArgs<T>& a, const BinArgs& bn, int nbz, cplx<T>* out, int64_t out_rot_stride,
                             const cplx<T>* tw, int batch, cudaStream_t st);

@@ -986,6 +986,8 @@ __global__ void __launch_bounds__(256) k_bin_count_yz(SpreadArgs<T> a, BinArgs b
     }
     const int rank = bin_rank(bn.count + (int64_t)b * bn.nbins, bin);
     bin_max(bn.cmax + (int64_t)b * bn.nbins, bin, cm);
+    // the bin's samples by 32-cell stretches of x, for the bound on its cells
+    bin_rank(bn.xcount + (int64_t)b * bn.nbins * SPREADX_XC, bin < 0 ? -1 : bin * SPREADX_XC + ((packed & 1023) >> 5));
     if (live) {
         const int64_t o = (int64_t)b * a.m + j;
         bn.bin_of[o] = bin;
@@ -1039,8 +1041,6 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
     constexpr int NB1 = LEN / plan_radix(LEN, 0);
     constexpr int NH = LEN / 2;
     constexpr int NWARP = NT / 32;
-    constexpr float MAGIC = 12582912.0f;  // 1.5 * 2^23
-    constexpr int MAGIC_BITS = 0x4B400000;
     extern __shared__ __align__(16) unsigned char sx_raw[];
     int* tre = reinterpret_cast<int*>(sx_raw);
     int* tim = tre + ROWS * px;
@@ -1055,14 +1055,9 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float2* outb = out + (int64_t)b * out_rot_stride;
     // the source bins (by - {0, 1}) x (bz - {0, 1}): two runs of sorted samples
-    // (neighbours along y are adjacent), and a bound on the tile's cells: taps below
-    // 2^21, a cell's sum (at most the sum of |c|, the weights being <= 1) below 2^30;
-    // each bin's count times its largest |component| of c (from the binning pass)
-    // bounds that sum
+    // (neighbours along y are adjacent)
     const int* off = bn.offset + (int64_t)b * (bn.nbins + 1);
-    const int* cmax = bn.cmax + (int64_t)b * bn.nbins;
     int run_lo[2] = {0, 0}, run_n[2] = {0, 0};
-    float mx = 0.f, sm = 0.f;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int zz = bz - k;
@@ -1070,11 +1065,26 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
         const int first = zz * nby + max(by - 1, 0), last = zz * nby + by;
         run_lo[k] = off[first];
         run_n[k] = off[last + 1] - run_lo[k];
-        for (int i = first; i <= last; ++i) {
-            const float cm = __int_as_float(cmax[i]);
-            mx = fmaxf(mx, cm);
-            sm += (float)(off[i + 1] - off[i]) * cm;
+    }
+    // Fixed point: the scale is the power of two that keeps every cell below 2^30.  A
+    // cell of x stretch k receives samples whose origin lies in stretches k and k - 1, the
+    // weights being <= 1; lane 8 i + k: source bin i, its count there times its
+    // largest |component| of c (from the binning pass).  The looser bound by a bin's
+    // whole count left taps 21 bits and the spectrum less exact than FP32 sums.
+    float cell_max;
+    {
+        const int yy = by - ((lane >> 3) & 1), zz = bz - (lane >> 4);
+        float v = 0.f;
+        if (yy >= 0 && zz >= 0) {
+            const int64_t bin = (int64_t)b * bn.nbins + zz * nby + yy;
+            v = (float)bn.xcount[bin * SPREADX_XC + (lane & 7)] * __int_as_float(bn.cmax[bin]);
         }
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        const float left = __shfl_up_sync(0xffffffffu, v, 1);
+        cell_max = v + ((lane & 7) ? left : 0.f);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) cell_max = fmaxf(cell_max, __shfl_xor_sync(0xffffffffu, cell_max, o));
     }
     const int total = run_n[0] + run_n[1];
     if (total == 0) {
@@ -1087,7 +1097,8 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
         }
         return;
     }
-    const float scale = tile_scale(mx, sm * 1.0001f);
+    const int e30 = 30 - (((__float_as_int(cell_max * 1.0001f) >> 23) & 255) - 126);
+    const float scale = cell_max > 0.f ? __int_as_float(min(max(127 + e30, 1), 254) << 23) : 1.f;
     const float inv_scale = 1.f / scale;  // a power of two: exact
     // entry `lane` of record t of the runs
     const float* recs = bn.rec + (int64_t)b * a.m * SX_REC + min(lane, SX_REC - 1);
@@ -1145,8 +1156,8 @@ __global__ void __launch_bounds__(SX_NT, 3) k_spread_x(SpreadArgs<float> a, BinA
             if (tap && rr < rows) {
                 w *= wx;
                 const int cell = base + o;
-                atomicAdd(tre + cell, __float_as_int(fmaf(cx, w, MAGIC)) - MAGIC_BITS);
-                atomicAdd(tim + cell, __float_as_int(fmaf(cy, w, MAGIC)) - MAGIC_BITS);
+                atomicAdd(tre + cell, __float2int_rn(cx * w));
+                atomicAdd(tim + cell, __float2int_rn(cy * w));
             }
         }
     }
@@ -2100,9 +2111,9 @@ cudaError_t launch_spread_x_t(const SpreadArgs<T>& a, const BinArgs& bn, int nbz
     if constexpr (sizeof(T) != 4) {
         return cudaErrorInvalidValue;
     } else {
-        if (a.w != SX_W || 2 * a.s > a.n_full) return cudaErrorInvalidValue;
-        // the counts and the bins' largest |c| components, adjacent in the workspace
-        cudaError_t e = cudaMemsetAsync(bn.count, 0, 2 * sizeof(int) * (size_t)batch * bn.nbins, st);
+        if (a.w != SX_W || 2 * a.s > a.n_full || a.s > 32 * SPREADX_XC) return cudaErrorInvalidValue;
+        // the counts, the bins' largest |c| components and the stretches' counts, adjacent in the workspace
+        cudaError_t e = cudaMemsetAsync(bn.count, 0, (2 + SPREADX_XC) * sizeof(int) * (size_t)batch * bn.nbins, st);
         if (e != cudaSuccess) return e;
         const dim3 gpts((unsigned)((a.m + 255) / 256), batch);
         if (a.m > 0) {
