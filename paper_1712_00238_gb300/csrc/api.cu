@@ -436,8 +436,11 @@ static int get_tw(sd_ctx* ctx, const Geo& G, Tw<T>* tw, cudaStream_t st) {
 // x pass: rows of the box
 template <typename T>
 static cudaError_t pass_x_fwd(const Geo& G, const Tw<T>& tw, const cplx<T>* in, int64_t in_rs, cplx<T>* out,
-                              int64_t out_rs, int batch, cudaStream_t st, int mode = ROW_FWD) {
+                              int64_t out_rs, int batch, cudaStream_t st, int mode = ROW_FWD, float ball = 0.f,
+                              float pad = 0.f) {
     RowArgs<T> r{};
+    r.ball = ball;
+    r.pad = pad;
     r.in = in;
     r.out = out;
     r.in_rot_stride = in_rs;
@@ -956,10 +959,6 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
     const bool iyx = S.cluster(), half = S.half();
     for (int64_t r0 = r_lo; r0 < r_hi; r0 += B) {
         const int b = (int)std::min<int64_t>(B, r_hi - r0);
-        if (!fused_x) {
-            PassTimer pt(ctx, SD_PASS_CLEAR, s, timed);
-            CK(ctx, cudaMemsetAsync(S.b0, 0, (size_t)b * S.e0 * sizeof(C), s));
-        }
         SpreadArgs<T> sa{};
         sa.pos = (const vec4<T>*)S.moving->pos;
         sa.c = (const C*)S.moving->c;
@@ -981,6 +980,14 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
         const int mx = pruned ? ROW_FWD_P : ROW_FWD;
         const int my = pruned ? COL_FWD_P : COL_FWD;
         const int mf = pruned ? COL_FUSED_P : COL_FUSED;
+        // clear and read only what the rotated taps reach
+        sa.ball = pruned && !fused_x && G.dim == 3 && G.n >= BALL_MIN_N ? fmaxf((float)(S.moving->radius * G.inv_h), 0.5f) : 0.f;
+        sa.pad = 0.5f * ctx->p.w + 1.f;
+        if (!fused_x) {
+            PassTimer pt(ctx, SD_PASS_CLEAR, s, timed);
+            if (sa.ball > 0.f) CK(ctx, launch_clear_ball<T>(sa, b, s));
+            else CK(ctx, cudaMemsetAsync(S.b0, 0, (size_t)b * S.e0 * sizeof(C), s));
+        }
         const C* Wp = half ? S.Wh[pruned] : (pruned ? S.Wsh : S.W);
         if (fused_x) {
             // spreading and the forward x transform in one pass: no sub-box
@@ -994,7 +1001,7 @@ static int search_enqueue(sd_ctx* ctx, const Search<T>& S, int64_t r_lo, int64_t
                 else CK(ctx, launch_spread<T>(sa, G.dim, b, s));
             }
             PassTimer pt(ctx, SD_PASS_FWD_X, s, timed);
-            CK(ctx, pass_x_fwd<T>(G, S.tw, S.b0, S.e0, S.b1, S.e1, b, s, mx));
+            CK(ctx, pass_x_fwd<T>(G, S.tw, S.b0, S.e0, S.b1, S.e1, b, s, mx, sa.ball, sa.pad));
         }
         C* fin;
         int64_t fin_rs;

@@ -9,7 +9,6 @@
 //                    column, so both products land on the same mode kz of one line,
 //                    G = W/2 FFT(x_c) + conj(W(-kappa))/2 FFT(conj x_c'), and one
 //                    inverse transform serves the two;
-//   inverse y        on N/2 columns (the ordinary pass);
 //   inverse y        on N/2 columns; its last stage holds outputs y and y + N/2 of a
 //                    column in one thread and writes them as the modes kappa and -kappa
 //                    of one complex line X = G_y + i G_(y + N/2), X(-kappa) = conj G_y + i conj G_(y + N/2)

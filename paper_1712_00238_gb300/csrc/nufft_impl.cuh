@@ -92,6 +92,35 @@ __device__ __forceinline__ int wrap_index(int a, int s) {
     return a < 0 ? a + s : a;
 }
 
+// Cells [lo, hi) along one axis of the sub-box that a rotated sample's taps can reach,
+// lo and hi even (s is), given the other axes' part of the distance (ball_dist2): the
+// samples lie in a ball of `ball` cells about cell s_h, a tap within half the kernel of
+// its sample along each axis; `pad` is that and one cell for the rounding of the rotation
+// and of the origin.  Empty (0, 0) if there are none.  The ball
+// is little more than half of its cube: the rest is neither cleared nor read.
+__device__ __forceinline__ float ball_dist2(float pad, int s_h, int i) {
+    const float d = fmaxf(fabsf((float)(i - s_h)) - pad, 0.f);
+    return d * d;
+}
+__device__ __forceinline__ void ball_range(float ball, float pad, int s, int s_h, float dist2, int* lo, int* hi) {
+    const float d2 = ball * ball - dist2;
+    const int reach = (int)(sqrtf(fmaxf(d2, 0.f)) + pad) + 1;
+    *lo = d2 < 0.f ? 0 : max(s_h - reach, 0) & ~1;
+    *hi = d2 < 0.f ? 0 : min((s_h + reach + 2) & ~1, s);
+}
+
+// A warp per row; bound by its stores (two cells of FP32, one of FP64 each).
+template <typename T>
+__global__ void __launch_bounds__(256) k_clear_ball(SpreadArgs<T> a) {
+    const int row = blockIdx.x * 8 + (int)(threadIdx.x >> 5);
+    if (row >= a.s * a.s) return;
+    int lo, hi;
+    ball_range(a.ball, a.pad, a.s, a.s_h, ball_dist2(a.pad, a.s_h, row % a.s) + ball_dist2(a.pad, a.s_h, row / a.s), &lo, &hi);
+    constexpr int V = sizeof(T) == 4 ? 2 : 1;
+    float4* q = reinterpret_cast<float4*>(a.out + blockIdx.y * a.out_rot_stride + (int64_t)row * a.s);
+    for (int i = lo / V + (int)(threadIdx.x & 31); i < hi / V; i += 32) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // Adds the taps of one sample to the sub-box with global atomics.  Along x the
 // six (or W) cells of a row are added two at a time with one 16-byte vector
 // atomic on an even-aligned cell pair (the out-of-row half of an edge pair adds
@@ -1383,7 +1412,8 @@ __global__ void __launch_bounds__(cta_threads<T, LENF>(), MB) k_cols_mb(ColArgs<
 __host__ __device__ constexpr int col_pitch(int len) { return len + 1; }
 
 // x pass: rows of the sub-box -> N modes per row (row stride N = LEN/2).
-template <typename T, int LEN>
+// BALL: of the rows only the cells within the ball are set.
+template <typename T, int LEN, bool BALL>
 __device__ __forceinline__ void rows_fwd_p_body(const RowArgs<T>& a) {
     using C = cplx<T>;
     constexpr int TR = lines_per_cta<T, LEN>();
@@ -1403,9 +1433,30 @@ __device__ __forceinline__ void rows_fwd_p_body(const RowArgs<T>& a) {
     const int nrows = a.nrows - row0;
     const int s = a.len_in;
     const C zero = mk(T(0), T(0));
+    // the cells of each line that are set (first | count << 16): worked out once a CTA,
+    // in every thread they took the pass from 556 to 747 us (12 rotations at N = 256)
+    __shared__ int cells[BALL ? TR : 1];
+    if constexpr (BALL) {
+        int lo = 0, hi = 0;
+        if ((int)threadIdx.x < TR) {
+            const int row = row0 + (int)threadIdx.x, z = row / s;
+            const float d2 = ball_dist2(a.pad, a.s_h, z) + ball_dist2(a.pad, a.s_h, row - z * s);
+            if ((int)threadIdx.x < nrows) ball_range(a.ball, a.pad, s, a.s_h, d2, &lo, &hi);
+            cells[threadIdx.x] = lo | (hi - lo) << 16;
+        }
+        if (!__syncthreads_or(hi)) {  // rows that no tap reaches
+            for (int j = threadIdx.x; j < min(TR, nrows) * NH; j += cta_threads<T, LEN>()) out[j] = zero;
+            return;
+        }
+    }
     auto load = [&](int line, int i, int r) -> C {
         const int pos = i + r * NB1;
-        return (line < nrows && pos < s) ? in[line * rs + pos] : zero;
+        if constexpr (BALL) {
+            const int c = cells[line];
+            return (unsigned)(pos - (c & 0xffff)) < (unsigned)(c >> 16) ? in[line * rs + pos] : zero;
+        } else {
+            return (line < nrows && pos < s) ? in[line * rs + pos] : zero;
+        }
     };
     auto emit = [&](int line, int i, int r, C v) {
         if (kept_out<LEN>(r) && line < nrows) out[line * NH + i + kept_slot<LEN>(r)] = v;
@@ -1414,9 +1465,9 @@ __device__ __forceinline__ void rows_fwd_p_body(const RowArgs<T>& a) {
                                                                                      LoadedHook([&] { tws.store(tw); }));
 }
 
-template <typename T, int LEN, int MB>
+template <typename T, int LEN, int MB, bool BALL>
 __global__ void __launch_bounds__(cta_threads<T, LEN>(), MB) k_rows_fwd_p(RowArgs<T> a) {
-    rows_fwd_p_body<T, LEN>(a);
+    rows_fwd_p_body<T, LEN, BALL>(a);
 }
 
 // y pass (3D): columns (one per kept x mode) of each z plane -> N modes, TC
@@ -1784,7 +1835,9 @@ static cudaError_t rows_fwd_p_impl(const RowArgs<T>& a, int batch, cudaStream_t 
     const int nb = (a.nrows + TR - 1) / TR;
     if (nb == 0 || batch == 0) return cudaSuccess;
     const size_t smem = (size_t)(TR * line_pitch(LEN) + tw_count(LEN)) * sizeof(C);
-    auto kern = k_rows_fwd_p<T, LEN, pruned_min_ctas<T, LEN, 0>()>;
+    auto kern = k_rows_fwd_p<T, LEN, pruned_min_ctas<T, LEN, 0>(), false>;
+    if constexpr (LEN >= BALL_MIN_N)
+        if (a.ball > 0.f) kern = k_rows_fwd_p<T, LEN, pruned_min_ctas<T, LEN, 0>(), true>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(nb, batch), cta_threads<T, LEN>(), smem, st>>>(a);
@@ -2277,6 +2330,12 @@ cudaError_t launch_interleave_t(const cplx<T>* src0, const cplx<T>* src1, cplx<T
                                                   cudaStream_t st) {                                    \
         return launch_spread_bins_t<T>(a, bn, dim, batch, st);                                          \
     }                                                                                                   \
+    template <> cudaError_t launch_clear_ball<T>(const SpreadArgs<T>& a, int batch, cudaStream_t st) {           \
+        if (a.s <= 0 || batch == 0) return cudaSuccess;                                                          \
+        k_clear_ball<T><<<dim3((a.s * a.s + 7) / 8, batch), 256, 0, st>>>(a);                                    \
+        note_launch();                                                                                           \
+        return cudaGetLastError();                                                                               \
+    }                                                                                                            \
     template <> cudaError_t launch_spread_x<T>(const SpreadArgs<T>& a, const BinArgs& bn, int nbz, cplx<T>* out, \
                                                int64_t ors, const cplx<T>* tw, int batch, cudaStream_t st) {   \
         return launch_spread_x_t<T>(a, bn, nbz, out, ors, tw, batch, st);                               \
