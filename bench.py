@@ -208,8 +208,18 @@ def host_inputs(w, torch):
     return {k: torch.from_numpy(np.ascontiguousarray(v)).pin_memory() for k, v in t.items()}
 
 
-def algorithmic_bytes_per_rotation(s: int, N: int, m_moving: int, dim: int = 3, c: int = 8) -> dict:
-    """Bytes each pass must move per rotation (complex elements of c bytes: 8 for complex64)."""
+def algorithmic_bytes_per_rotation(s: int, N: int, m_moving: int, dim: int = 3, c: int = 8,
+                                   half: bool = False) -> dict:
+    """Bytes each pass must move per rotation (complex elements of c bytes: 8 for complex64).
+    half: the passes after the product work on half the spectrum (searches that keep Re f_N alone)."""
+    if half:
+        b = algorithmic_bytes_per_rotation(s, N, m_moving, dim, c)
+        vol = N ** dim
+        b["fused"] -= vol * c // 2  # the product table is whole, the output half
+        b["inv_x"] = vol * c // 2
+        if dim == 3:
+            b["inv_y"] = vol * c
+        return b
     if dim == 2:
         return {
             "clear": s * s * c,
@@ -384,8 +394,9 @@ def run_ours(args):
     # roofline of the dominant search pass (live CUDA-event times of the timed steps)
     radius = float(np.linalg.norm(w.moving.query.pos, axis=1).max())
     s = sub_box(radius, w.N, w.L, w.w)
-    per_rot = algorithmic_bytes_per_rotation(s, w.N, w.moving.query.m, w.dim, 16 if w.precision == "f64" else 8)
     passes = {k: v for k, v in ptimes.items() if v[0] > 0 and k != "graph"}
+    half = "inv_yx" not in passes  # the cluster inverse works on whole planes
+    per_rot = algorithmic_bytes_per_rotation(s, w.N, w.moving.query.m, w.dim, 16 if w.precision == "f64" else 8, half)
     roofline = None
     pass_report = {}
     l2_resident = w.dim == 2  # a few MB per rotation: the passes run out of L2, HBM does not bound them
@@ -402,7 +413,7 @@ def run_ours(args):
         avg_s = t * 1e-3 / n
         peak, src = measured_peak()
         ach = per_launch / avg_s / 1e9
-        traffic = traffic_per_launch(dom, s, w.N, plan_used.get("batch"))
+        traffic = traffic_per_launch(dom + "_half" if half else dom, s, w.N, plan_used.get("batch"))
         roofline = {"bound": "hbm", "kernel": dom, "achieved": round(ach, 1), "peak": peak, "unit": "GB/s",
                     "frac": round(ach / peak, 4), "peak_source": src,
                     "algorithmic_bytes_per_launch": int(per_launch),
@@ -517,10 +528,15 @@ FFT_PLAN_TEXT = {
 # DRAM once per launch (the launch's other rotations hit L2), the rest scales
 # with the rotations.  Peg-in-bore: one 34-rotation launch read 552,969,728 B and
 # wrote 529,623,040 B; its W' (16.8 MB) stays mostly in L2, so the model is per
-# rotation only.  A pass of another shape reports null.
+# rotation only.  "fused_half" is the fused pass with the half-spectrum output: one
+# 20-rotation docking launch read 985,174,272 B and wrote 535,934,464 B, one of 34
+# peg-in-bore rotations 539,886,592 and 260,166,912.  A pass of
+# another shape reports null.
 TRAFFIC_MODEL: dict = {
     ("fused", 156, 192): ((976803840 - 56623104 + 1081333248) / 20, 56623104),
     ("fused", 108, 128): ((552969728 + 529623040) / 34, 0),
+    ("fused_half", 108, 128): ((539886592 + 260166912) / 34, 0),
+    ("fused_half", 156, 192): ((985174272 - 56623104 + 535934464) / 20, 56623104),
 }
 
 
@@ -785,7 +801,7 @@ def run_pairs(args):
     alg = 0.0
     for w, (fx, mv, _, g) in zip(mine, jobs):
         sb = sub_box(mv.radius, w.N, w.L, w.w)
-        alg += n_rot * sum(algorithmic_bytes_per_rotation(sb, w.N, mv.m).values())
+        alg += n_rot * sum(algorithmic_bytes_per_rotation(sb, w.N, mv.m, half=True).values())
     peak, peak_kind = measured_peak()
     achieved = alg / (ms * 1e-3) / 1e9
     result = {
