@@ -247,9 +247,8 @@ __global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_inv_min_ctas<T, LE
 
 // A row pass leaves this many CTAs per SM before its CTAs take more groups, up to a
 // most each: the copies then run ahead, and a K-best merge (K block-wide rounds) is
-// paid once.  68 rotations at N = 128: 161 us without bulk copies, 148 with; 60 at
-// N = 192: 521 -> 461 (with one comparison per butterfly where each output took one);
-// 77 at N = 96 keeping four: 174 -> 133 (8 CTAs per SM, 32 groups; 160 at 16 and 16).
+// paid once.  (77 rotations at N = 96 keeping four: 133 us at 8 CTAs per SM and 32
+// groups, 160 at 16 and 16.)
 template <int K>
 __host__ __device__ constexpr int half_row_wave() { return K == 1 ? 16 : 8; }
 template <int K>
@@ -261,39 +260,23 @@ __host__ __device__ constexpr int rows_half_min_ctas() { return K == 1 ? 4 : (K 
 
 // Inverse x of packed lines.  Row groups of TR lines (2 TR rows) are handled by one
 // CTA in turn: its K best are kept in registers across the groups and merged once.
-// Whether a row pass's groups come in by bulk copies (two-stage FP32 lines; an FP64
+// Whether a row pass's groups are copied in ahead (two-stage FP32 lines; an FP64
 // CTA's raw lines would cost it its shared memory).
 template <typename T, int LEN>
-__host__ __device__ constexpr bool rows_half_bulk() {
+__host__ __device__ constexpr bool rows_half_ahead() {
     return sizeof(T) == 4 && plan_radix(LEN, 1) != 0;
 }
 template <typename T, int LEN, int K>
 __host__ __device__ constexpr size_t rows_half_smem() {
     constexpr int TR = lines_per_cta<T, LEN>(), NT = cta_threads<T, LEN>();
-    return (size_t)(TR * ((rows_half_bulk<T, LEN>() ? LEN : 0) + line_pitch(LEN)) + tw_count(LEN)) * sizeof(cplx<T>) +
+    return (size_t)(TR * ((rows_half_ahead<T, LEN>() ? LEN : 0) + line_pitch(LEN)) + tw_count(LEN)) * sizeof(cplx<T>) +
            (K > 1 ? (size_t)NT * K * (sizeof(T) + sizeof(int)) : 0);
 }
 
-// One bulk copy (bytes and both addresses multiples of 16) that reports to an
-// mbarrier, and the bounded wait for its phase.
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst), b = (unsigned)__cvta_generic_to_shared(bar);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d), "l"(src),
-                 "r"(bytes), "r"(b)
-                 : "memory");
-}
-__device__ __forceinline__ bool bulk_wait(uint64_t* bar, unsigned phase) {
-    const unsigned b = (unsigned)__cvta_generic_to_shared(bar);
-    for (int tries = 0; tries < (1 << 22); ++tries) {
-        unsigned ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok)
-                     : "r"(b), "r"(phase)
-                     : "memory");
-        if (ok) return true;
-    }
-    return false;
+// Sixteen bytes from global to shared memory without a register and past L1.
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 
 __device__ __forceinline__ float max_num(float a, float b) { return fmaxf(a, b); }
@@ -308,31 +291,25 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
     constexpr int NTW = tw_count(LEN);
     constexpr int NB1 = LEN / plan_radix(LEN, 0);
     constexpr int RL = plan_last_radix(LEN), PL = LEN / RL;
-    constexpr bool BULK = rows_half_bulk<T, LEN>();
+    constexpr bool AHEAD = rows_half_ahead<T, LEN>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* raw = reinterpret_cast<C*>(smem_raw);
-    C* buf = raw + (BULK ? TR * LEN : 0);
+    C* buf = raw + (AHEAD ? TR * LEN : 0);
     C* tw = buf + TR * LD;
     constexpr int NH = LEN / 2;
     const C* in = a.in + (int64_t)blockIdx.y * a.in_rot_stride;
     const int nlines = a.nrows / 2, ngroups = (nlines + TR - 1) / TR;
-    // a group's lines are contiguous: one bulk copy brings the next group in while this
-    // one is in its second stage
-    __shared__ __align__(8) uint64_t bar;
+    // a group's lines are contiguous (and a line is a multiple of 16 bytes): the CTA's
+    // threads copy the next group in while this one is in its second stage
     auto fetch = [&](int g) {
-        if (g < ngroups)
-            bulk_copy(raw, in + (int64_t)g * TR * LEN, (unsigned)(min(TR, nlines - g * TR) * LEN * sizeof(C)), &bar);
-    };
-    if constexpr (BULK) {
-        if (threadIdx.x == 0) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&bar)) : "memory");
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            fetch(blockIdx.x);
+        if (g < ngroups) {
+            const int quads = min(TR, nlines - g * TR) * (int)(LEN * sizeof(C) / 16);
+            const float4* src = reinterpret_cast<const float4*>(in + (int64_t)g * TR * LEN);
+            for (int t = threadIdx.x; t < quads; t += NT) copy_async16(reinterpret_cast<float4*>(raw) + t, src + t);
         }
-        __syncthreads();
-    }
-    unsigned phase = 0;
-    bool lost = false;
+        copy_commit();
+    };
+    if constexpr (AHEAD) fetch(blockIdx.x);
     TwStage<C, NTW, NT> tws;
     tws.load(a.tw);
     const C zero = mk(T(0), T(0));
@@ -345,12 +322,12 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
         const int line0 = g * TR;
         const int nl = nlines - line0;
         const C* src = in + (int64_t)line0 * LEN;
-        if constexpr (BULK) {
-            lost |= !bulk_wait(&bar, phase);  // (a copy that never came: the CTA finds nothing)
-            phase ^= 1;
+        if constexpr (AHEAD) {  // every thread's share has landed
+            copy_wait();
+            __syncthreads();
         }
         auto load = [&](int line, int i, int r) -> C {
-            return line < nl ? (BULK ? raw : src)[line * LEN + i + r * NB1] : zero;
+            return line < nl ? (AHEAD ? raw : src)[line * LEN + i + r * NB1] : zero;
         };
         // a butterfly's outputs are kept until all are there: one maximum each, and the
         // comparisons with what the thread holds only where that maximum could enter it
@@ -394,15 +371,10 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
                     if (g == (int)blockIdx.x) tws.store(tw);
                 },
                 [&] {
-                    if (BULK && threadIdx.x == 0) fetch(g + gridDim.x);
+                    if constexpr (AHEAD) fetch(g + gridDim.x);
                 }));
         // the next group's first writes to buf come after the barrier that follows
         // this group's last reads
-    }
-    if (BULK && lost) {
-        bestA = bestB = -INFINITY;
-        idxA = idxB = INT_MAX;
-        if constexpr (K > 1) top.init();
     }
     if constexpr (K > 1) {
         T* sv = reinterpret_cast<T*>(tw + NTW);
