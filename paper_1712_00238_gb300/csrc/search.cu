@@ -58,7 +58,7 @@ __device__ __forceinline__ Cand load_cand(const Cand* p) {
 // skipped, and the selection ends when what is left of the k fills its bucket.  A
 // few reads of the list by one SM, whatever k is (54,000 candidates, k = 100: 5.06 ms
 // for k arg-best passes).  Shared memory: the k selected keys, then sorted.
-constexpr int TOPK_THREADS = 1024;
+constexpr int TOPK_THREADS = 1024, TOPK_MAX = 4096;
 
 __global__ void __launch_bounds__(TOPK_THREADS) k_topk(const Cand* cand, int64_t n, int k, Cand* out) {
     extern __shared__ __align__(16) unsigned char tk_raw[];
@@ -185,9 +185,12 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk(const Cand* cand, int64_t
 cudaError_t launch_topk(const void* cand, int64_t n, int k, void* out, cudaStream_t st) {
     int p2 = 1;
     while (p2 < k) p2 <<= 1;
-    const size_t smem = (size_t)p2 * (2 * sizeof(unsigned long long) + sizeof(unsigned));
+    constexpr size_t key = 2 * sizeof(unsigned long long) + sizeof(unsigned);
+    const size_t smem = (size_t)p2 * key;
     if (smem > 32 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // one value per kernel and device, always that of the largest k: a call on
+        // another thread must not lower it between this one's setting and its launch
+        const cudaError_t e = cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TOPK_MAX * key));
         if (e != cudaSuccess) return e;
     }
     k_topk<<<1, TOPK_THREADS, smem, st>>>(reinterpret_cast<const Cand*>(cand), n, k, reinterpret_cast<Cand*>(out));
