@@ -294,17 +294,21 @@ __global__ void __launch_bounds__(RS_TILE) k_rescore_move(RescoreArgs<T> a) {
 constexpr int RS_QUEUE = 256;  // pair slots per warp
 constexpr int RS_EXP = 256;    // entries of the table
 
-// exp(-r2 / (2 s^2)) from r2 and k = 256 / (2 s^2 ln 2); 0 <= r2 k < 2^18.
+// exp(-r2 / (2 s^2)) from r2 and k = 256 / (2 s^2 ln 2), r2 k >= 0.  The screen's FP32
+// coordinates may lie a whole cutoff off where positions exceed s by their 24 bits, so
+// any r2 can come: past 2^-1000 (m in the low word, the high word magic's own) the
+// result is 0, by integer tests that take nothing from the FP64 pipe.
 __device__ __forceinline__ double gauss_exp(double r2, double k, const double* tab) {
     const double magic = 6755399441055744.0;  // 1.5 * 2^52: the low word receives round(x)
     const double t = fma(r2, k, magic);
-    const int m = __double2loint(t);
+    const unsigned m = (unsigned)__double2loint(t);
     const double f = fma(r2, k, magic - t);
     static_assert(RS_EXP == 1 << 8, "");
     constexpr double c = -0.6931471805599453094 / RS_EXP;
     const double q = f * fma(f, fma(f, fma(f, c * c * c * c / 24.0, c * c * c / 6.0), c * c / 2.0), c);
     const double w = tab[m & (RS_EXP - 1)];
-    const double e = __hiloint2double(__double2hiint(w) - ((m >> 8) << 20), __double2loint(w));
+    const bool in = __double2hiint(t) == 0x43380000 && m < 1000u * RS_EXP;
+    const double e = __hiloint2double(in ? __double2hiint(w) - (int)((m >> 8) << 20) : 0, in ? __double2loint(w) : 0);
     return fma(e, q, e);
 }
 
