@@ -890,6 +890,33 @@ static int search_setup(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* movi
     return SD_OK;
 }
 
+// The stream on which to make what outlives the call: the caller's, or while that is
+// being captured one of its own (memory allocated on a captured stream belongs to the
+// graph, and what fills it would run at its replays only).
+struct KeepStream {
+    cudaStream_t st;
+    cudaError_t err = cudaSuccess;
+    explicit KeepStream(cudaStream_t caller) : st(caller) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(caller, &cap) != cudaSuccess) cudaGetLastError();
+        if (cap != cudaStreamCaptureStatusActive) return;
+        own = true;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        err = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    }
+    // before the caller's stream uses what was made
+    cudaError_t join() { return own ? cudaStreamSynchronize(st) : cudaSuccess; }
+    ~KeepStream() {
+        if (!own) return;
+        if (err == cudaSuccess) cudaStreamDestroy(st);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+
+private:
+    bool own = false;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // the thread's own while swapped
+};
+
 // The product table that a job's plan reads, made on the stream if the fixed shape
 // has not met this grid and sub-box yet.
 template <typename T>
@@ -903,9 +930,16 @@ static int search_tables(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
     for (auto& w : cache)
         if (w.first == s_h) ws = w.second;
     if (!ws) {
-        CK(ctx, pool_alloc(&ws, (size_t)S->Nd * sizeof(cplx<T>), st));
-        if (half) CK(ctx, launch_whalf<T>(S->W, S->G.N, S->G.dim, S->G.n, s_h, (cplx<T>*)ws, st));
-        else CK(ctx, launch_wshift<T>(S->W, S->G.N, S->G.dim, S->G.n, s_h, (cplx<T>*)ws, st));
+        KeepStream keep(st);
+        CK(ctx, keep.err);
+        CK(ctx, pool_alloc(&ws, (size_t)S->Nd * sizeof(cplx<T>), keep.st));
+        cudaError_t e = half ? launch_whalf<T>(S->W, S->G.N, S->G.dim, S->G.n, s_h, (cplx<T>*)ws, keep.st)
+                             : launch_wshift<T>(S->W, S->G.N, S->G.dim, S->G.n, s_h, (cplx<T>*)ws, keep.st);
+        if (e == cudaSuccess) e = keep.join();
+        if (e != cudaSuccess) {
+            pool_free(ws, keep.st);
+            CK(ctx, e);
+        }
         cache.emplace_back(s_h, ws);
     }
     if (half) S->Wh[pruned] = (const cplx<T>*)ws;
