@@ -550,10 +550,14 @@ def launch_count() -> int:
 
 
 def decode_cands(buf: torch.Tensor):
-    """(score float64, rot int32, idx int32) of a candidate buffer (views of one copy of it)."""
-    b = buf.reshape(-1, CAND_BYTES).clone(memory_format=torch.contiguous_format)
-    ri = b.view(torch.int32)
-    return b.view(torch.float64)[:, 0], ri[:, 2], ri[:, 3]
+    """(score float64, rot int32, idx int32) of a candidate buffer: one copy of it, scores first (contiguous)."""
+    b = buf.reshape(-1, CAND_BYTES)
+    if b.data_ptr() % 8 or b.storage_offset() % 8 or b.stride() != (CAND_BYTES, 1):
+        b = b.clone(memory_format=torch.contiguous_format)
+    n = b.shape[0]
+    w = b.view(torch.float64).t().clone(memory_format=torch.contiguous_format)
+    ri = w.view(torch.int32)
+    return w[0], ri.as_strided((n,), (2,), 2 * n), ri.as_strided((n,), (2,), 2 * n + 1)
 
 
 # ---------------------------------------------------------------------------
