@@ -155,8 +155,8 @@ const char* sd_last_error(const sd_ctx* ctx);
  * default 0), "spread_fused" (1: in
  * pruned 3D FP32 searches with w = 6, spread each rotation's samples straight
  * into whole rows held in shared memory and run the forward x transform there,
- * with no sub-box in device memory, as long as a batch's 108 bytes per sample and
- * rotation stay below 7 GB; default 0), "sdf_cull" (2, the default:
+ * with no sub-box in device memory, as long as a batch's workspace, 108 bytes per
+ * sample and rotation and its bin tables, stays within 7 GiB; default 0), "sdf_cull" (2, the default:
  * the SDF sums skip every 256-sample boundary tile that lies beyond the
  * truncation radius (1 + eps)|xi| of every query of a block, and each warp skips
  * the 32-sample sub-tiles beyond that radius of its own 32 queries -- the

@@ -832,10 +832,13 @@ struct Search {
     int nbz = 0;  // SPREAD_X: bins along z
 };
 
-// A batch's records of fused spreading (108 bytes a sample and rotation with the bins)
-// stay below 7 GB; larger jobs spread directly.
+// The workspace of fused spreading (108 bytes a sample and rotation, and the bin tables)
+// stays within 7 GiB a batch; larger jobs spread as without it.
+constexpr size_t SPREAD_X_MAX = (size_t)7 << 30;
 template <typename T>
-static bool spread_x_fits(const Search<T>& S, int batch) { return S.moving->m * batch <= (int64_t)1 << 26; }
+static bool spread_x_fits(const Search<T>& S, int batch) {
+    return bins_bytes_x(S.G.s, S.moving->m, batch) <= SPREAD_X_MAX;
+}
 
 // Spreading fused with the x transform: pruned 3D FP32 searches with w = 6.
 template <typename T>
@@ -859,6 +862,24 @@ static int fft_plan_default(const sd_ctx* ctx, const Search<T>& S) {
     return S.prunable ? SD_FFT_PRUNED : SD_FFT_FULL;
 }
 
+// The spreading a job starts from at its plan's batch (may be fused if `fused`).
+template <typename T>
+static int bins_default(const sd_ctx* ctx, const Search<T>& S, bool fused) {
+    if (fused && ctx->opt_spread_fused && spread_x_ok(ctx, S, S.plan.B)) return SPREAD_X;
+    if (!bins_supported(ctx)) return 0;
+    return ctx->opt_spread_box ? SPREAD_BOX : (ctx->opt_spread_direct ? 0 : ctx->opt_bin_side);
+}
+
+// A tuned or imported plan in place of the default one, as far as it applies.
+template <typename T>
+static void adopt_plan(const sd_ctx* ctx, Search<T>* S, const Plan& tuned) {
+    S->plan.B = (int)std::min<int64_t>(tuned.B, std::max<int64_t>(S->n_r, 1));
+    if (tuned.bins != SPREAD_X) S->plan.bins = tuned.bins;
+    else if (spread_x_fits(*S, S->plan.B)) S->plan.bins = SPREAD_X;
+    else S->plan.bins = bins_default(ctx, *S, false);  // also where the default batch would have fitted
+    if (ctx->opt_fft_plan < 0 && fft_plan_ok(*S, tuned.fft)) S->plan.fft = tuned.fft;
+}
+
 // Fixed-shape tables, geometry, twiddles and the default plan of a job (may
 // synchronise the stream the first time a fixed shape meets a grid).
 template <typename T>
@@ -875,7 +896,6 @@ static int search_setup(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* movi
     S->out = out;
     S->maps = maps;
     S->plan.B = choose_batch<T>(ctx, S->G, n_r);
-    S->plan.bins = (!ctx->opt_spread_direct && bins_supported(ctx)) ? ctx->opt_bin_side : 0;
     per_rot_elems<T>(S->G, &S->e0, &S->e1);
     S->rows_last = (S->G.dim == 2) ? S->G.N : (int64_t)S->G.N * S->G.N;
     S->Nd = (S->G.dim == 2) ? (int64_t)S->G.N * S->G.N : (int64_t)S->G.N * S->G.N * S->G.N;
@@ -885,8 +905,7 @@ static int search_setup(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* movi
     S->prep = prep;
     S->plan.fft = fft_plan_default(ctx, *S);
     S->iyx = ctx->opt_inv_cluster && sizeof(T) == 4 && S->G.dim == 3 && inv_yx_supported(S->G.N);
-    if (ctx->opt_spread_box && bins_supported(ctx)) S->plan.bins = SPREAD_BOX;
-    if (ctx->opt_spread_fused && spread_x_ok(ctx, *S, S->plan.B)) S->plan.bins = SPREAD_X;
+    S->plan.bins = bins_default(ctx, *S, true);
     return SD_OK;
 }
 
@@ -1118,9 +1137,7 @@ static int autotune(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
     const std::string key = plan_key(ctx, *S);
     auto it = ctx->tuned.find(key);
     if (it != ctx->tuned.end()) {
-        S->plan.B = (int)std::min<int64_t>(it->second.B, std::max<int64_t>(S->n_r, 1));
-        if (it->second.bins != SPREAD_X || spread_x_fits(*S, S->plan.B)) S->plan.bins = it->second.bins;
-        if (ctx->opt_fft_plan < 0 && fft_plan_ok(*S, it->second.fft)) S->plan.fft = it->second.fft;
+        adopt_plan(ctx, S, it->second);
         return SD_OK;
     }
     // first stage: batch x spreading under the job's default FFT plan; second
@@ -1749,19 +1766,13 @@ int sd_search_plan(sd_ctx* ctx, const sd_shape* moving, const sd_grid* g, int64_
         S.moving = moving;
         S.n_r = n_r;
         S.plan.B = choose_batch<T>(ctx, S.G, n_r);
-        S.plan.bins = (!ctx->opt_spread_direct && bins_supported(ctx)) ? ctx->opt_bin_side : 0;
         S.prunable = ctx->opt_pruned && pruned_len_ok(S.G.n) && S.G.s <= S.G.N;
         S.alt_cols = S.prunable && sizeof(T) == 4 && S.G.n >= 128 && S.G.n <= 384;
         S.plan.fft = fft_plan_default(ctx, S);
-        if (ctx->opt_spread_box && bins_supported(ctx)) S.plan.bins = SPREAD_BOX;
-        if (ctx->opt_spread_fused && spread_x_ok(ctx, S, S.plan.B)) S.plan.bins = SPREAD_X;
+        S.plan.bins = bins_default(ctx, S, true);
         if (ctx->opt_autotune && !ctx->opt_plain && ctx->opt_batch <= 0) {
             auto it = ctx->tuned.find(plan_key(ctx, S));
-            if (it != ctx->tuned.end()) {
-                S.plan.B = (int)std::min<int64_t>(it->second.B, n_r);
-                if (it->second.bins != SPREAD_X || spread_x_fits(S, S.plan.B)) S.plan.bins = it->second.bins;
-                if (ctx->opt_fft_plan < 0 && fft_plan_ok(S, it->second.fft)) S.plan.fft = it->second.fft;
-            }
+            if (it != ctx->tuned.end()) adopt_plan(ctx, &S, it->second);
         }
         if (batch) *batch = S.plan.B;
         if (spread_bins) *spread_bins = S.plan.bins;
