@@ -453,7 +453,7 @@ int sd_refine(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* moving, const 
  *          number of candidates have rot = idx = -1
  * Scratch: none beyond the selection kernel's shared memory, so calls on any
  * streams or threads are independent.  Larger inputs return SD_ERR_ARG.
- * Cost: one CTA reads the candidates a few times (once per byte in which they
+ * Cost: one CTA reads the candidates k times (k <= 3) or a few (once per byte in which they
  * differ, until k are fixed) and sorts k keys.
  * Asynchronous on `stream`. */
 int sd_top_k_static(sd_ctx* ctx, const sd_cand* cand, int64_t n_cand, int k, sd_cand* out, void* stream);

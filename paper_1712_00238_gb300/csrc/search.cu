@@ -3,7 +3,8 @@
 //
 // top-k: one CTA finds the k-th candidate in the order (score descending, rotation
 // ascending, translation index ascending, position) by radix selection, collects
-// the k that do not come after it and sorts them in shared memory.
+// the k that do not come after it and sorts them in shared memory; up to three
+// candidates take an arg-best pass each.
 // re-score: f_c(R, t) = sum_ij c1_i c2_j G_{sigma_g sqrt 2}(R p2_j + t - p1_i) in
 // FP64 (the continuous score of Eq. 8 for Gaussian-represented SDFs).  Pairs
 // are screened in FP32 against a cutoff of 8 sigma_g sqrt 2 (with a margin), and
@@ -53,13 +54,53 @@ __device__ __forceinline__ Cand load_cand(const Cand* p) {
     return c;
 }
 
+constexpr int TOPK_THREADS = 1024, TOPK_MAX = 4096;
+
+// Up to three candidates take a pass each: the first in the order after the one before.
+// The selection below reads the list at least three times and counts its bytes.  Passes
+// against the selection, us a call: k = 1 of 54,000 candidates 74 against 205, of 2^20
+// 641 against 2,760; k = 2 110 against 232 and 1,257 against 3,370; k = 3 (by the two
+// above: 36 and 620 a pass) about 146 against 185 and 1,880 against 3,370; at k = 4 they
+// are even.
+constexpr int TOPK_PASSES = 3;
+
+__global__ void __launch_bounds__(TOPK_THREADS) k_topk_passes(const Cand* cand, int64_t n, int k, Cand* out) {
+    __shared__ CandKey won[TOPK_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const CandKey none{~0ull, ~0ull, ~0u};  // after every candidate: no position is 2^32 - 1
+    CandKey prev{0, 0, 0};
+    for (int it = 0; it < k; ++it) {
+        CandKey best = none;
+#pragma unroll 4
+        for (int64_t p = tid; p < n; p += TOPK_THREADS) {
+            const CandKey q = cand_key(load_cand(cand + p), p);
+            if (key_less(q, best) && (it == 0 || key_less(prev, q))) best = q;
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            const CandKey o{__shfl_xor_sync(0xffffffffu, best.a, off), __shfl_xor_sync(0xffffffffu, best.b, off),
+                            __shfl_xor_sync(0xffffffffu, best.c, off)};
+            if (key_less(o, best)) best = o;
+        }
+        if (lane == 0) won[warp] = best;
+        __syncthreads();
+        for (int w = 0; w < TOPK_THREADS / 32; ++w)
+            if (key_less(won[w], best)) best = won[w];
+        __syncthreads();
+        if (tid == 0) {
+            Cand c;
+            if (best.c != none.c) c = load_cand(cand + best.c);
+            else { c.score = -INFINITY; c.rot = -1; c.idx = -1; }
+            out[it] = c;
+        }
+        prev = best;
+    }
+}
+
 // Radix selection a byte of the key at a time, most significant first, over the
 // candidates that share the bytes fixed so far; bytes equal in all of them are
 // skipped, and the selection ends when what is left of the k fills its bucket.  A
 // few reads of the list by one SM, whatever k is (54,000 candidates, k = 100: 5.06 ms
 // for k arg-best passes).  Shared memory: the k selected keys, then sorted.
-constexpr int TOPK_THREADS = 1024, TOPK_MAX = 4096;
-
 __global__ void __launch_bounds__(TOPK_THREADS) k_topk(const Cand* cand, int64_t n, int k, Cand* out) {
     extern __shared__ __align__(16) unsigned char tk_raw[];
     __shared__ int hist[256];
@@ -183,6 +224,11 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk(const Cand* cand, int64_t
 }
 
 cudaError_t launch_topk(const void* cand, int64_t n, int k, void* out, cudaStream_t st) {
+    if (k <= TOPK_PASSES) {
+        k_topk_passes<<<1, TOPK_THREADS, 0, st>>>(reinterpret_cast<const Cand*>(cand), n, k, reinterpret_cast<Cand*>(out));
+        note_launch();
+        return cudaGetLastError();
+    }
     int p2 = 1;
     while (p2 < k) p2 <<= 1;
     constexpr size_t key = 2 * sizeof(unsigned long long) + sizeof(unsigned);
