@@ -17,7 +17,8 @@
 // finishing kernel combines the partials in a fixed order, so the results do
 // not depend on how many CTAs shared the work's scheduling.
 // In 3D both passes walk the boundary as a two-level tree instead (256-sample tiles
-// of 32-sample sub-tiles, the Morton order's own hierarchy): see k_sdf_tree.
+// of 32-sample sub-tiles, the Morton order's own hierarchy): see k_sdf_tree; small
+// builds' distances and memberships take all pairs (sdf_tree_pays).
 #include <float.h>
 #include <math.h>
 
@@ -37,8 +38,8 @@ __device__ __forceinline__ T recip(T x) { return T(1) / x; }
 template <>
 __device__ __forceinline__ float recip<float>(float x) { return __frcp_rn(x); }
 
-// 2D: every pair.
-template <typename T>
+// Every pair: 2D, and 3D builds too small for the tree (sdf_tree_pays).
+template <typename T, int D>
 __global__ void __launch_bounds__(SDF_TILE) k_sdf_nearest(SdfArgs<T> a, int tiles_per_split, T* part_d2, T* part_w) {
     __shared__ vec4<T> sq[SDF_TILE];
     __shared__ vec4<T> sn[SDF_TILE];  // normal with the area in .w
@@ -59,14 +60,20 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_nearest(SdfArgs<T> a, int tile
             sn[threadIdx.x] = a.nrm[j];
         }
         __syncthreads();
-        const int cnt = (int)min((int64_t)SDF_TILE, a.n_b - t0);
+        const int cnt = live ? (int)min((int64_t)SDF_TILE, a.n_b - t0) : 0;
         for (int k = 0; k < cnt; ++k) {
             const vec4<T> q = sq[k];
             const vec4<T> nn = sn[k];
-            const T dx = q.x - p.x, dy = q.y - p.y;
-            const T d2 = dx * dx + dy * dy;
+            const T dx = q.x - p.x, dy = q.y - p.y, dz = D == 3 ? q.z - p.z : T(0);
+            const T d2 = dx * dx + dy * dy + dz * dz;
             dmin = d2 < dmin ? d2 : dmin;
-            wind += nn.w * (dx * nn.x + dy * nn.y) * recip(d2);
+            const T dot = dx * nn.x + dy * nn.y + dz * nn.z;
+            if (D == 3) {
+                const T r = rsqrt(d2);
+                wind += nn.w * dot * r * r * r;
+            } else {
+                wind += nn.w * dot * recip(d2);
+            }
         }
         __syncthreads();
     }
@@ -77,7 +84,7 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_nearest(SdfArgs<T> a, int tile
 
 // Nearest distance (the smallest partial) and membership (the partial winding
 // sums added in split order) of each query.
-template <typename T>
+template <typename T, int D>
 __global__ void k_sdf_nearest_finish(SdfArgs<T> a, int splits, const T* part_d2, const T* part_w) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.m) return;
@@ -87,7 +94,7 @@ __global__ void k_sdf_nearest_finish(SdfArgs<T> a, int splits, const T* part_d2,
         dmin = d < dmin ? d : dmin;
         wind += part_w[(int64_t)k * a.m + i];
     }
-    const T S = T(2.0 * M_PI);
+    const T S = D == 3 ? T(4.0 * M_PI) : T(2.0 * M_PI);
     a.xi_abs[i] = sqrt(dmin);
     int8_t m = (wind > T(0.5) * S) ? int8_t(-1) : int8_t(1);
     if (a.pmc_override) {
@@ -916,7 +923,7 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_skin(SdfArgs<T> a) {
 }
 
 // Boundary-tile splits per query block: enough CTAs for about four per SM.
-static int sdf_splits(int64_t query_blocks, int64_t tiles) {
+static int sdf_splits(int64_t query_blocks, int64_t tiles, int most = 64) {
     static int sms = 0;
     if (!sms) {
         int dev = 0;
@@ -926,25 +933,45 @@ static int sdf_splits(int64_t query_blocks, int64_t tiles) {
     }
     int64_t s = (4 * (int64_t)sms + query_blocks - 1) / query_blocks;
     s = s < 1 ? 1 : (s > tiles ? tiles : s);
-    return (int)(s > 64 ? 64 : s);
+    return (int)(s > most ? most : s);
+}
+
+// Whether the tree is faster than all pairs for nearest distances and memberships.  The
+// tree's CTAs walk the whole boundary for 32 or 64 queries each (90 us for 5,000 samples,
+// 1 ms for 300,000), so it takes queries enough to fill the GPU, and boundary enough to
+// leave out; all pairs cost their number and split the boundary too.  The lines lie where
+// builds of 1 to 50,000 queries (a cube and a band about a sphere of 100 to 300,000
+// samples) change sides.  FP32, us a build by tree / pairs: 500 queries, 20,000 samples
+// 346 / 220; 500, 300,000 1,109 / 450; 50,000, 1,000 267 / 242; 5,000, 20,000 366 / 329;
+// 10,000, 20,000 391 / 415; 50,000, 5,000 365 / 452.  FP64 (the pair costs ten times as
+// much, and so do the tree's nodes): 500, 5,000 1,335 / 540; 50,000, 300 1,334 / 960;
+// 5,000, 5,000 1,329 / 1,280; 10,000, 5,000 1,731 / 2,830.
+template <typename T>
+static bool sdf_tree_pays(int64_t m, int64_t n_b) {
+    return sizeof(T) == 4 ? (m - 3300) * n_b > 60000000 : (m - 500) * n_b > 25000000;
 }
 
 // Nearest distances and memberships: the tree in 3D (its nodes, and the list of
-// queries left to the full sum), all pairs in 2D.
+// queries left to the full sum), all pairs in 2D and in small builds.
 template <typename T>
 static cudaError_t launch_nearest(const SdfArgs<T>& a, int dim, cudaStream_t st) {
     const unsigned nb = (unsigned)((a.m + SDF_TILE - 1) / SDF_TILE);
     char* scratch = nullptr;
     cudaError_t e;
-    if (dim == 2) {
+    if (dim == 2 || !sdf_tree_pays<T>(a.m, a.n_b)) {
         const int64_t tiles = (a.n_b + SDF_TILE - 1) / SDF_TILE;
-        const int splits = sdf_splits(nb, tiles < 1 ? 1 : tiles);
+        const int splits = sdf_splits(nb, tiles < 1 ? 1 : tiles, dim == 2 ? 64 : 256);
         const int tps = (int)((tiles + splits - 1) / splits);
         if ((e = pool_alloc((void**)&scratch, (size_t)2 * splits * a.m * sizeof(T), st)) != cudaSuccess) return e;
         T* d2 = reinterpret_cast<T*>(scratch);
         T* w = d2 + (size_t)splits * a.m;
-        k_sdf_nearest<T><<<dim3(nb, splits), SDF_TILE, 0, st>>>(a, tps, d2, w);
-        k_sdf_nearest_finish<T><<<nb, SDF_TILE, 0, st>>>(a, splits, d2, w);
+        if (dim == 2) {
+            k_sdf_nearest<T, 2><<<dim3(nb, splits), SDF_TILE, 0, st>>>(a, tps, d2, w);
+            k_sdf_nearest_finish<T, 2><<<nb, SDF_TILE, 0, st>>>(a, splits, d2, w);
+        } else {
+            k_sdf_nearest<T, 3><<<dim3(nb, splits), SDF_TILE, 0, st>>>(a, tps, d2, w);
+            k_sdf_nearest_finish<T, 3><<<nb, SDF_TILE, 0, st>>>(a, splits, d2, w);
+        }
         note_launch(2);
     } else {
         const size_t nodes_bytes = (size_t)a.n_tiles * (1 + SDF_TILE / 32) * NODE * sizeof(T);
