@@ -22,6 +22,8 @@
 #include <float.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace sd {
@@ -744,9 +746,11 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_sum(SdfArgs<T> a, int tiles_pe
 // (1 + eps) max|xi|, each warp taking one of a tile's sub-tiles unless it lies beyond
 // every lane's own reach: what is skipped holds no pair that passes Eq. 17t.  What a lane adds, and in which order, does not depend on what
 // is skipped.  (One CTA per 256 queries, in lock-step over whole tiles: 14.0 ms for
-// 5,000 spheres.)
+// 5,000 spheres.)  Queries too few to fill the GPU have the tiles dealt to several CTAs
+// (grid y, sum_splits; in turn, as a group's near tiles are neighbours), a partial sum
+// each with its compensation, which k_sdf_sum_finish adds.
 template <typename T>
-__global__ void __launch_bounds__(32 * TREE_NW) k_sdf_sum_tree(SdfArgs<T> a) {
+__global__ void __launch_bounds__(32 * TREE_NW) k_sdf_sum_tree(SdfArgs<T> a, cplx<T>* part) {
     constexpr int SUB = SDF_TILE / 32;
     __shared__ T sh[4][TREE_NW][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -770,14 +774,14 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_sum_tree(SdfArgs<T> a) {
     const T inv_2s2 = recip(T(2) * a.sigma * a.sigma);
     const T xi2 = xi * xi;
     T sr = 0, cr = 0, si = 0, ci = 0;
-    const int n_tiles = (int)a.n_tiles;
-    for (int base = 0; base < n_tiles; base += 32) {
-        const int t = base + lane;
+    const int step = (int)gridDim.y, n_tiles = (int)a.n_tiles;
+    for (int base = (int)blockIdx.y; base < n_tiles; base += 32 * step) {
+        const int t = base + lane * step;
         // NaN reach (a query whose distance is none) keeps every tile
         const bool in = t < n_tiles && !(a.tile_box && box_gap2(a.tile_box + (int64_t)t * 6, lo, hi) > reach2);
         unsigned m = __ballot_sync(0xffffffffu, in);
         while (m) {
-            const int tt = base + __ffs(m) - 1;
+            const int tt = base + (__ffs(m) - 1) * step;
             m &= m - 1;
             const int64_t j0 = (int64_t)tt * SDF_TILE + warp * 32;
             const int cnt = (int)min((int64_t)32, a.n_b - j0);
@@ -815,6 +819,11 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_sum_tree(SdfArgs<T> a) {
         kahan_add(si, ci, sh[2][w][lane]);
         kahan_add(si, ci, -sh[3][w][lane]);
     }
+    if (part) {
+        part[2 * ((int64_t)blockIdx.y * a.m + i)] = mk(sr, si);
+        part[2 * ((int64_t)blockIdx.y * a.m + i) + 1] = mk(cr, ci);
+        return;
+    }
     const T v = a.vol[src];
     a.c_out[i] = mk(sr * v, si * v);
     if (a.rho_out) a.rho_out[src] = mk(sr, si);
@@ -823,17 +832,21 @@ __global__ void __launch_bounds__(32 * TREE_NW) k_sdf_sum_tree(SdfArgs<T> a) {
     a.pos_out[i] = po;
 }
 
-// rho of each query: the partial sums added in split order (compensated), then
-// the shape's sample c = rho v and position.
-template <typename T>
+// rho of each query: the partial sums added in split order (compensated; PAIRS: with the
+// partials' own compensations), then the shape's sample c = rho v and position.
+template <typename T, bool PAIRS>
 __global__ void k_sdf_sum_finish(SdfArgs<T> a, int splits, const cplx<T>* part) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.m) return;
     T sr = 0, cr = 0, si = 0, ci = 0;
     for (int k = 0; k < splits; ++k) {
-        const cplx<T> v = part[(int64_t)k * a.m + i];
-        kahan_add(sr, cr, v.x);
-        kahan_add(si, ci, v.y);
+        const cplx<T>* p = part + ((int64_t)k * a.m + i) * (PAIRS ? 2 : 1);
+        kahan_add(sr, cr, p[0].x);
+        kahan_add(si, ci, p[0].y);
+        if constexpr (PAIRS) {
+            kahan_add(sr, cr, -p[1].x);
+            kahan_add(si, ci, -p[1].y);
+        }
     }
     const int64_t src = a.perm_q ? (int64_t)a.perm_q[i] : i;
     const T v = a.vol[src];
@@ -936,6 +949,16 @@ static int sdf_splits(int64_t query_blocks, int64_t tiles, int most = 64) {
     return (int)(s > most ? most : s);
 }
 
+// Splits of the boundary's tiles for `groups` groups of 32 queries in the truncated sum:
+// 16 CTAs a SM in all (8 and 32 within 15 % either way, 32 more for the finishing to
+// add), a split with at least four tiles.  FP32, us a build without / with: 500 queries
+// about 20,000 samples 1,107 / 290 (in a cube; 525 / 290 in a band at the boundary),
+// 2,000 about 300,000 14,190 / 1,880 (3,600 / 1,230); FP64, 500 about 5,000 3,420 / 1,140.
+static int sum_splits(int64_t groups, int64_t tiles) {
+    const int64_t s = std::min((16 * 152 + groups - 1) / groups, std::min<int64_t>(tiles / 4, 256));
+    return s < 1 ? 1 : (int)s;
+}
+
 // Whether the tree is faster than all pairs for nearest distances and memberships.  The
 // tree's CTAs walk the whole boundary for 32 or 64 queries each (90 us for 5,000 samples,
 // 1 ms for 300,000), so it takes queries enough to fill the GPU, and boundary enough to
@@ -1026,8 +1049,17 @@ cudaError_t launch_sdf(const SdfArgs<T>& a, int dim, cudaStream_t st) {
         return cudaGetLastError();
     }
     if (dim == 3 && a.phi == SD_PHI_SDF && a.eps >= T(0)) {
-        k_sdf_sum_tree<T><<<(unsigned)((a.m + 31) / 32), 32 * TREE_NW, 0, st>>>(a);
+        const int64_t groups = (a.m + 31) / 32;
+        const int splits = sum_splits(groups, a.n_tiles);
+        cplx<T>* part = nullptr;
+        if (splits > 1 && (e = pool_alloc((void**)&part, (size_t)splits * a.m * 2 * sizeof(cplx<T>), st)) != cudaSuccess) return e;
+        k_sdf_sum_tree<T><<<dim3((unsigned)groups, splits), 32 * TREE_NW, 0, st>>>(a, part);
         note_launch();
+        if (part) {
+            k_sdf_sum_finish<T, true><<<nb, SDF_TILE, 0, st>>>(a, splits, part);
+            note_launch();
+            pool_free(part, st);
+        }
         return cudaGetLastError();
     }
     // every pair (no truncation, or 2D): the boundary tiles of a query block split
@@ -1054,7 +1086,7 @@ cudaError_t launch_sdf(const SdfArgs<T>& a, int dim, cudaStream_t st) {
             break;
     }
 #undef SD_SUM
-    k_sdf_sum_finish<T><<<nb, SDF_TILE, 0, st>>>(a, splits, part);
+    k_sdf_sum_finish<T, false><<<nb, SDF_TILE, 0, st>>>(a, splits, part);
     note_launch(2);
     pool_free(part, st);
     return cudaGetLastError();

@@ -71,3 +71,33 @@ def test_few_queries_take_all_pairs(m, precision):
         assert (r[:, 0].double() - g(xi / 0.8 - 1)).abs().max() < tol
         assert (r[:, 1].double() - 3 * g(xi / 0.8 + 1)).abs().max() < tol
     ctx.close()
+
+
+# splits of the truncated sum: 16 x 152 CTAs shared out among groups of 32 queries, four tiles a split
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("n_b,m", [(2047, 40), (2048, 40), (2304, 33), (20001, 1), (20001, 700), (70000, 300)])
+def test_split_sums_match_full_sums(n_b, m, precision):
+    rng = np.random.default_rng(np.random.SeedSequence([n_b, m, 33]))
+    real = np.float32 if precision == "f32" else np.float64
+    eps = np.finfo(real).eps
+    for kind in ("closed", "open"):
+        pos, nrm, area = _boundary(kind, n_b, rng)
+        qry = _queries(m, rng)
+        pos, nrm, area, qry = (x.astype(real) for x in (pos, nrm, area, qry))
+        dist, w, rho, mag = _reference(qry, pos, nrm, area)
+        sure = (w - 0.5).abs() > (1e-4 if n_b < 50000 else 1e-3)
+        ctx = sd.Context(3, precision, 0, sigma_g=0.1)
+        n0 = sd.launch_count()
+        _, r = ctx.sdf_build(pos, nrm, area, qry, np.ones(m), return_rho=True)
+        launches = sd.launch_count() - n0
+        got = torch.view_as_complex(r)
+        tol = 100 * eps * mag.amax() + 30 * eps * rho.abs().amax()
+        assert ((got - rho).abs()[sure] <= tol + _edge_terms(qry, pos, nrm, area, dist, eps)[sure]).all()
+        ctx.set_option("sdf_cull", 0)
+        _, r0 = ctx.sdf_build(pos, nrm, area, qry, np.ones(m), return_rho=True)
+        assert torch.equal(torch.view_as_complex(r0), got)  # what the boxes leave out adds nothing
+        # the launches of a build whose boundary is too small to split, and one that adds the splits
+        n0 = sd.launch_count()
+        ctx.sdf_build(pos[:1000], nrm[:1000], area[:1000], qry, np.ones(m))
+        assert launches == sd.launch_count() - n0 + 1
+        ctx.close()
