@@ -404,7 +404,7 @@ int sd_score_grad(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* moving, co
  *   trans  device, P x 3 real (updated in place; 2D: z ignored)
  *   hist   device, (steps + 1) x P real, or NULL: the score before each step
  *          and after the last
- * Asynchronous on `stream`; one gather and one small kernel per step. */
+ * Asynchronous on `stream`; one launch per step for few poses, a gather and a small kernel for many. */
 int sd_refine_poses(sd_ctx* ctx, const sd_shape* fixed, const sd_shape* moving, const sd_grid* g,
                     void* quats, void* trans, int64_t P, int steps, double lr_t, double lr_q, void* hist,
                     void* stream);

@@ -91,12 +91,11 @@ __device__ __forceinline__ void rotate_left(double q[4], const double th[3]) {
 //   dynamics:  v <- (1 - gamma) v + h F / m, w <- (1 - gamma) w + h T / I,
 //              t += h v, q <- exp(h w) q.
 // state (P x 12 doubles): CG (gF, gT, dF, dT) of the previous step; dynamics (v, w).
-// One warp; the ascent's divisions go to its lanes (serial FP64 division is most of
-// the update's time), the other rules run on lane 0.
-template <typename T>
+// WARP: one warp a pose; the ascent's divisions go to its lanes (serial FP64 division is
+// most of the update's time), the other rules run on lane 0.  Else one thread a pose.
+template <typename T, bool WARP>
 __device__ __forceinline__ void refine_update(const double a[7], int64_t p, int dim, const RefineParams& rp, T* quats,
                                               T* trans, double* state, int first) {
-    const int lane = threadIdx.x & 31;
     T* qo = quats + 4 * p;
     T* to = trans + 3 * p;
     double q[4] = {qo[0], qo[1], qo[2], qo[3]};
@@ -114,8 +113,16 @@ __device__ __forceinline__ void refine_update(const double a[7], int64_t p, int 
         double sf = 1e-30, sq = 1e-30;
         for (int k = 0; k < 3; ++k) sf = fmax(sf, fabs(F[k]));
         for (int k = 0; k < 4; ++k) sq = fmax(sq, fabs(dq[k]));
+        if constexpr (!WARP) {
+            double qn[4];
+            for (int k = 0; k < 4; ++k) qn[k] = q[k] + rp.lr_q * dq[k] / sq;
+            const double nn = sqrt(qn[0] * qn[0] + qn[1] * qn[1] + qn[2] * qn[2] + qn[3] * qn[3]);
+            for (int k = 0; k < 4; ++k) qo[k] = (T)(nn > 0 ? qn[k] / nn : qn[k]);
+            for (int k = 0; k < dim; ++k) to[k] = (T)(t[k] + rp.lr_t * F[k] / sf);
+            return;
+        }
         // lanes 0-3: a quaternion entry each, lanes 4-6: a translation entry
-        const int k = lane & 3;
+        const int lane = threadIdx.x & 31, k = lane & 3;
         const bool is_t = (lane & 4) != 0;
         const double cur = is_t ? (k == 0 ? t[0] : (k == 1 ? t[1] : t[2]))
                                 : (k == 0 ? q[0] : (k == 1 ? q[1] : (k == 2 ? q[2] : q[3])));
@@ -129,7 +136,7 @@ __device__ __forceinline__ void refine_update(const double a[7], int64_t p, int 
         else if (lane < 4 + dim) to[k] = (T)moved;
         return;
     }
-    if (lane != 0) return;
+    if (WARP && (threadIdx.x & 31) != 0) return;
     if (rp.method == SD_REFINE_CG) {
         const double* g[2] = {F, Tq};
         double d[2][3];
@@ -190,9 +197,30 @@ __device__ __noinline__ void finish_pose(const GatherArgs<T>& a, int pose) {
     if (lane < 8) __stcg(sums + lane, 0.0);
     if (a.step) {
         if (a.hist && lane == 0) a.hist[pose] = (T)f[0];
-        if (!a.last) refine_update<T>(f, pose, D, a.rp, a.quats_io, a.trans_io, a.state, a.first);
+        if (!a.last) refine_update<T, true>(f, pose, D, a.rp, a.quats_io, a.trans_io, a.state, a.first);
     } else if (lane == 0) {
         grad_finish<T>(f, pose, D, a.quats, a.score, a.dq, a.dt);
+    }
+}
+
+// The same by one thread a pose, in a launch of its own, after gathers of many CTAs
+// (launch_gather): there the update's FP64 chain in every pose's last CTA, and the 64
+// registers that its call holds in all of them, cost more than a launch.
+template <typename T>
+__global__ void __launch_bounds__(32) k_finish_poses(GatherArgs<T> a, int dim) {
+    const int64_t pose = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    if (pose >= a.P) return;
+    double f[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        f[k] = a.acc[8 * pose + k];
+        a.acc[8 * pose + k] = 0.0;
+    }
+    if (a.step) {
+        if (a.hist) a.hist[pose] = (T)f[0];
+        if (!a.last) refine_update<T, false>(f, pose, dim, a.rp, a.quats_io, a.trans_io, a.state, a.first);
+    } else {
+        grad_finish<T>(f, pose, dim, a.quats, a.score, a.dq, a.dt);
     }
 }
 
@@ -205,7 +233,7 @@ __device__ __noinline__ void finish_pose(const GatherArgs<T>& a, int pose) {
 // and accumulates score, force and torque over its samples; lanes and warps are
 // summed in FP64 and added to the pose's accumulators.  The CTA that adds the last
 // share of a pose finishes it (gradient outputs, or the pose's update) and clears the
-// accumulators for the next launch, so a refinement step is one launch: 57 us with a
+// accumulators for the next launch, so a refinement step of few poses is one launch: 57 us with a
 // clearing and an update launch of its own and 256 samples per CTA, at 10 poses x
 // 2,280 samples, 26 now.  Few poses take fewer samples per CTA (a.chunk), so many that
 // one wave of four CTAs per SM holds them all: eight CTAs per SM took 34 us a step,
@@ -415,9 +443,10 @@ __device__ __forceinline__ void warp_sums(const T acc[7], double* out) {
     if ((lane & 3) == 0 && (lane >> 2) < 7) out[lane >> 2] = v[0];
 }
 
-// (64 registers: four CTAs per SM.)
-template <typename T, int D, int W>
-__global__ void __launch_bounds__(GA_THREADS, sizeof(T) == 4 && W <= 6 ? 4 : 0) k_gather(GatherArgs<T> a) {
+// APART: k_finish_poses finishes the poses.  (With finish_pose 64 registers: four CTAs per
+// SM; without, 37 to 48 in most forms, and five to six.)
+template <typename T, int D, int W, bool APART>
+__global__ void __launch_bounds__(GA_THREADS, sizeof(T) == 4 && W <= 6 && !APART ? 4 : 0) k_gather(GatherArgs<T> a) {
     constexpr int NWARP = GA_THREADS / 32;
     __shared__ T stage[gather_chunk<T, D, W>() * gather_rec<D, W>()];
     __shared__ double red[NWARP][7];
@@ -428,10 +457,26 @@ __global__ void __launch_bounds__(GA_THREADS, sizeof(T) == 4 && W <= 6 ? 4 : 0) 
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     T Rm[9], tv[3];
-    pose_matrix<T, D>(a.quats + 4 * (int64_t)pose, a.trans + 3 * (int64_t)pose, Rm, tv);
+    if constexpr (sizeof(T) == 4) {
+        pose_matrix<T, D>(a.quats + 4 * (int64_t)pose, a.trans + 3 * (int64_t)pose, Rm, tv);
+    } else {  // FP64 by one warp: eight would queue for the pipe
+        __shared__ T pm[12];
+        if (threadIdx.x < 32) {
+            pose_matrix<T, D>(a.quats + 4 * (int64_t)pose, a.trans + 3 * (int64_t)pose, Rm, tv);
+            if (threadIdx.x == 0) {
+                for (int k = 0; k < 9; ++k) pm[k] = Rm[k];
+                for (int k = 0; k < 3; ++k) pm[9 + k] = tv[k];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 9; ++k) Rm[k] = pm[k];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) tv[k] = pm[9 + k];
+    }
     const int64_t j0 = (int64_t)blockIdx.x * a.chunk;
     const int nj = (int)((a.m2 - j0) < (int64_t)a.chunk ? (a.m2 - j0) : (int64_t)a.chunk);
-    gather_stage<T, D, W, GA_THREADS>(a, Rm, tv, j0, nj, a.chunk <= GA_THREADS / 4, stage);
+    gather_stage<T, D, W, GA_THREADS>(a, Rm, tv, j0, nj, a.few, stage);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     T acc[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
@@ -442,8 +487,9 @@ __global__ void __launch_bounds__(GA_THREADS, sizeof(T) == 4 && W <= 6 ? 4 : 0) 
         double s = 0.0;
         for (int w = 0; w < NWARP; ++w) s += red[w][threadIdx.x];
         atomicAdd(a.acc + 8 * (int64_t)pose + threadIdx.x, s);
-        __threadfence();  // before the count below
+        if (!APART) __threadfence();  // before the count below
     }
+    if constexpr (APART) return;
     __syncthreads();
     if (warp != 0) return;
     double* sums = a.acc + 8 * (int64_t)pose;
@@ -459,12 +505,26 @@ template <typename T>
 cudaError_t launch_gather(const GatherArgs<T>& args, int dim, cudaStream_t st) {
     if (args.P == 0 || args.m2 == 0) return cudaSuccess;
     GatherArgs<T> a = args;
-    // samples per CTA: at most what its stage holds, at least one per warp
-        constexpr int64_t CTAS = 4 * 152;  // one wave
+    constexpr int64_t CTAS = 4 * 152;  // one wave
+    bool apart = false;
+    // Samples per CTA: at most what its stage holds, at least one per warp, the wave's CTAs
+    // shared out evenly among the poses (512 poses x 50 samples in chunks of 48 took a second
+    // CTA each for two samples: FP64 in 2D 191 us a gradient, 105 now).
+    // Four threads a sample shorten the stage's latency but spend a lane in four (in 2D two)
+    // on no weight: not where the FP64 pipe is what bounds it (400 samples x 64 poses in 2D
+    // 116 us with, 100 without; in 3D 20 samples x 200 poses 62 with, 88 without).
+    // Poses are finished apart beyond two waves of CTAs (FP64: one), us a refinement of 20
+    // steps with finishing inside / apart: 2,000 poses x 130 samples in 2D by CG 2,118 / 1,100
+    // (a step kernel always: 1,533), x 2,000 in 2D 9,160 / 7,920; 512 x 400 in 3D at w = 8
+    // (1,024 CTAs) 5,340 / 5,740, FP64 in 2D 14,520 / 13,700.
     auto grid = [&](int most) {
-        const int64_t want = (a.m2 * a.P / CTAS + 7) / 8 * 8;
+        const int64_t per_pose = a.P < CTAS ? CTAS / a.P : 1;
+        const int64_t want = ((a.m2 + per_pose - 1) / per_pose + 7) / 8 * 8;
         a.chunk = (int)(want < 8 ? 8 : (want > most ? most : want));
-        return dim3((unsigned)((a.m2 + a.chunk - 1) / a.chunk), (unsigned)a.P);
+        const unsigned ctas = (unsigned)((a.m2 + a.chunk - 1) / a.chunk);
+        a.few = a.chunk <= GA_THREADS / 4 && (sizeof(T) == 4 || dim == 3 || ctas * a.P <= 152);
+        apart = ctas * a.P > (sizeof(T) == 4 ? 2 : 1) * CTAS;
+        return dim3(ctas, (unsigned)a.P);
     };
     // the second and later steps of a refinement may be set up while the previous runs
     cudaLaunchAttribute attr[1];
@@ -484,13 +544,17 @@ cudaError_t launch_gather(const GatherArgs<T>& args, int dim, cudaStream_t st) {
     case WW:                                                                                        \
         if (dim == 2) {                                                                             \
             const dim3 g = grid(gather_chunk<T, 2, WW>());                                          \
-            e = launch(k_gather<T, 2, WW>, g);                                                      \
+            e = launch(apart ? k_gather<T, 2, WW, true> : k_gather<T, 2, WW, false>, g);            \
         } else {                                                                                    \
             const dim3 g = grid(gather_chunk<T, 3, WW>());                                          \
-            e = launch(k_gather<T, 3, WW>, g);                                                      \
+            e = launch(apart ? k_gather<T, 3, WW, true> : k_gather<T, 3, WW, false>, g);            \
         }                                                                                           \
         note_launch();                                                                              \
-        return e != cudaSuccess ? e : cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();                                               \
+        if (e != cudaSuccess || !apart) return e;                                                   \
+        k_finish_poses<T><<<(unsigned)((a.P + 31) / 32), 32, 0, st>>>(a, dim);                      \
+        note_launch();                                                                              \
+        return cudaGetLastError();
     switch (a.w) {
         SD_GATHER_CASE(4) SD_GATHER_CASE(5) SD_GATHER_CASE(6) SD_GATHER_CASE(7) SD_GATHER_CASE(8)
         SD_GATHER_CASE(10) SD_GATHER_CASE(12) SD_GATHER_CASE(16)

@@ -296,7 +296,8 @@ struct GatherArgs {
     int w;
     double* acc;              // P x 8 (sums, CTAs done), zero before a launch and after it
     int chunk;                // samples per CTA (set by launch_gather)
-    // what the last CTA of a pose does: write the gradient ...
+    bool few;                 // four threads stage a sample (set by launch_gather)
+    // what the last CTA of a pose, or a launch after, does: write the gradient ...
     T* score;                 // P
     T* dq;                    // P x 4
     T* dt;                    // P x 3
