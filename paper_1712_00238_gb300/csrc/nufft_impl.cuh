@@ -2056,17 +2056,25 @@ cudaError_t launch_cols_t(int mode, const ColArgs<T>& a, int batch, cudaStream_t
     return cudaErrorInvalidValue;
 }
 
-// Samples in a launch up to which direct spreading takes eight lanes per sample: 12
-// rotations of 1,500 samples 28 -> 23 us, 13 of 2,280 29 -> 28; 64 of 2,280 (146 thousand)
-// are bound by the L2 atomics either way.
-constexpr int64_t SPREAD_LANES_MAX = 65536;
+// Samples in a launch up to which direct spreading takes eight lanes per sample: the
+// lanes shorten what one thread does in series, until the atomics bound both, and FP64
+// also pays for the 8 - w weights that no tap has.  us by one thread / eight lanes: FP32
+// w = 6 in 3D 18,000 samples 28.5 / 22.4, 48,000 55.1 / 40.8, 65,000 97.5 / 98.2 (w = 8:
+// 188 / 238); in 2D, whose threads have a row for a plane, 18,000 11.2 / 10.1, 48,000
+// 16.2 / 18.3; FP64 w = 4 6,000 49 / 30, 18,000 51 / 51, 32,000 53 / 86 in 3D; w = 6 in
+// 2D 18,000 42 / 34, 60,000 83 / 96; w = 8 in 2D 48,000 106 / 83.
+template <typename T>
+constexpr int64_t spread_lanes_max(int dim, int w) {
+    if (sizeof(T) == 8) return w < 6 ? 16000 : (dim == 2 && w < 8 ? 20000 : 60000);
+    return dim == 2 ? 20000 : 60000;
+}
 
 template <typename T>
 cudaError_t launch_spread_t(const SpreadArgs<T>& a, int dim, int batch, cudaStream_t st) {
     if (a.m == 0 || batch == 0) return cudaSuccess;
     const dim3 grid((unsigned)((a.m + 255) / 256), batch);
     const dim3 grid8((unsigned)((a.m + 31) / 32), batch);
-    const bool lanes = a.m * batch <= SPREAD_LANES_MAX;
+    const bool lanes = a.m * batch <= spread_lanes_max<T>(dim, a.w);
 #define SD_SPREAD_LANES(WW)                                                                  \
     if (lanes && a.w == WW) {                                                                \
         auto kern = (dim == 2) ? k_spread_lanes<T, 2, WW> : k_spread_lanes<T, 3, WW>;        \
