@@ -24,6 +24,7 @@ SOURCES = ["api.cu", "sdf.cu", "nufft_f32.cu", "nufft_f64.cu", "nufft_half_f32.c
            "topk_static.cu", "order.cu", "octree.cu", "peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + INCLUDE,
+         "-Xptxas", "-v",           # registers and spills of every kernel, kept beside the objects
          "-diag-suppress", "1444"]  # 1444: deprecated vector types in CUDA headers
 
 
@@ -63,6 +64,8 @@ def build(force: bool = False, jobs: int | None = None, verbose: bool = False) -
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stderr[-4000:]}")
+        with open(obj.replace(".o", ".ptxas"), "w") as f:
+            f.write(r.stderr)
         if verbose and r.stderr:
             print(r.stderr)
         return obj

@@ -1725,7 +1725,10 @@ __host__ __device__ constexpr int fused_std_min_ctas() {
 // for FP32 lines of 128 to 384 points: the narrow plan takes half the columns
 // per CTA (twice the CTAs, half the shared memory each, 64-byte row segments),
 // the wide plan twice (256-byte row segments, up to 99 KB of shared memory).
-// Their register bound keeps the per-thread cap of the standard plan.
+// Their register bound keeps the per-thread cap of the standard plan, but for the wide
+// 384-point passes: 256 threads of three radix-16 butterflies each spilled up to 1.2 KB at
+// its 64 registers, and shared memory allows two CTAs a SM at most, so two (128 registers;
+// 60 rotations at N = 192: forward y 1,643 -> 814 us, fused 5,481 -> 3,325).
 template <typename T, int LEN>
 __host__ __device__ constexpr bool alt_cols_ok() {
     return sizeof(T) == 4 && LEN >= 128 && LEN <= 384;
@@ -1736,6 +1739,7 @@ __host__ __device__ constexpr int alt_lines() {
 }
 template <typename T, int LEN, int KIND, int WIDE>
 __host__ __device__ constexpr int alt_min_ctas() {
+    if (WIDE && LEN == 384) return 2;
     return pruned_min_ctas<T, LEN, KIND>() * cta_threads<T, LEN>() / cta_threads_for<LEN>(alt_lines<T, LEN, WIDE>());
 }
 
