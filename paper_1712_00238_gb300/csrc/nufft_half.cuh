@@ -253,10 +253,23 @@ template <int K>
 __host__ __device__ constexpr int half_row_wave() { return K == 1 ? 16 : 8; }
 template <int K>
 __host__ __device__ constexpr int half_row_most() { return K == 1 ? 16 : 32; }
-// Register bound of the row pass: the two rows' running best take it past the 40
-// registers of six CTAs (192 points spilled: 247 us per 20 rotations against 175 at four).
-template <int K>
-__host__ __device__ constexpr int rows_half_min_ctas() { return K == 1 ? 4 : (K <= 4 ? 5 : 0); }
+// Resident CTAs a SM the row pass is compiled for (0: the compiler's choice): a bound
+// only where it measured faster, us of the pass without a bound / as chosen.  FP32, one
+// candidate: four, 64 registers (64 rotations at N = 128 148 / 144), but 192 points spill
+// under it (60 rotations 516 at four / 457).  Two: none (60 at 192 858 at five / 605).
+// Four: five at 96 points (64 rotations 131 / 106), four at 192 (60: 1,089 / 962).  More
+// keep their lists in registers.  FP64 two, below 64 points three: the pipe bounds it, and
+// the compiler's own 110 to 150 registers leave 192 points one CTA (15 rotations 3,166 /
+// 2,999) and 48 points two (48 rotations 154 / 137); elsewhere they are even, where four
+// and five spilled up to 3 KB (128 points keeping two 1,067 / 1,022).
+template <typename T, int LEN, int K>
+__host__ __device__ constexpr int rows_half_min_ctas() {
+    if (K > 4) return 0;
+    if (sizeof(T) == 8) return LEN < 64 ? 3 : 2;
+    if (K == 1) return LEN == 192 ? 0 : 4;
+    if (K == 4) return LEN == 96 ? 5 : (LEN == 192 ? 4 : 0);
+    return 0;
+}
 
 // Inverse x of packed lines.  Row groups of TR lines (2 TR rows) are handled by one
 // CTA in turn: its K best are kept in registers across the groups and merged once.
@@ -399,7 +412,7 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
 }
 
 template <typename T, int LEN, int K>
-__global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_half_min_ctas<K>())
+__global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_half_min_ctas<T, LEN, K>())
 k_rows_half(RowArgs<T> a) {
     rows_half_body<T, LEN, K>(a);
 }

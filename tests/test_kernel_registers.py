@@ -42,3 +42,11 @@ def _named(spills, pattern):
 def test_wide_plan_does_not_spill(spills, pattern):
     bad = {k: v for k, v in _named(spills, pattern).items() if v}
     assert not bad, bad
+
+
+def test_row_pass_of_the_searches_does_not_spill(spills):
+    # (precision, points, candidates kept) -> bytes that measured faster than a looser bound
+    allowed = {("f", 192, 4): 400, ("d", 192, 1): 150, ("d", 192, 2): 150, ("d", 192, 4): 800}
+    for name, n in _named(spills, r"k_rows_halfI[fd]Li\d+ELi\d+E").items():
+        t, length, keep = re.search(r"k_rows_halfI([fd])Li(\d+)ELi(\d+)E", name).groups()
+        assert n <= allowed.get((t, int(length), int(keep)), 64), (name, n)
