@@ -44,3 +44,14 @@ def _check(N, precision, reach, plan, rotations):
 @pytest.mark.parametrize("plan", [0, 1, 2, 3])
 def test_plans_of_384_points(plan):
     _check(192, "f32", 0.6, plan, 2)
+
+
+# reach 0.6: the sub-box fits half a line; 2.4: it does not (full passes; their tables exceed 32 MB at 192 and 256)
+@pytest.mark.parametrize("precision,N,reach,rotations", [("f32", 128, 0.6, 2), ("f32", 128, 2.4, 2), ("f32", 192, 2.4, 1),
+                                                         ("f32", 256, 0.6, 2), ("f32", 256, 2.4, 1), ("f64", 128, 0.6, 2),
+                                                         ("f64", 128, 2.4, 1), ("f64", 192, 0.6, 1), ("f64", 192, 2.4, 1),
+                                                         ("f64", 256, 0.6, 1), ("f64", 256, 2.4, 1)])
+def test_long_lines(precision, N, reach, rotations):
+    _check(N, precision, reach, 1 if reach < 1 else 0, rotations)
+    if reach < 1:
+        _check(N, precision, reach, 0, rotations)
