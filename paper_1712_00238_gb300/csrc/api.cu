@@ -874,10 +874,11 @@ static int bins_default(const sd_ctx* ctx, const Search<T>& S, bool fused) {
 template <typename T>
 static void adopt_plan(const sd_ctx* ctx, Search<T>* S, const Plan& tuned) {
     S->plan.B = (int)std::min<int64_t>(tuned.B, std::max<int64_t>(S->n_r, 1));
-    if (tuned.bins != SPREAD_X) S->plan.bins = tuned.bins;
-    else if (spread_x_fits(*S, S->plan.B)) S->plan.bins = SPREAD_X;
-    else S->plan.bins = bins_default(ctx, *S, false);  // also where the default batch would have fitted
     if (ctx->opt_fft_plan < 0 && fft_plan_ok(*S, tuned.fft)) S->plan.fft = tuned.fft;
+    // fused spreading writes what the pruned 3D passes read: only where this job, at this
+    // batch and forward plan, can run it (also where the default batch would have fitted)
+    if (tuned.bins != SPREAD_X) S->plan.bins = tuned.bins;
+    else S->plan.bins = spread_x_ok(ctx, *S, S->plan.B) ? SPREAD_X : bins_default(ctx, *S, false);
 }
 
 // Fixed-shape tables, geometry, twiddles and the default plan of a job (may
