@@ -1163,6 +1163,7 @@ static int autotune(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
     Plan best = S->plan;
     double best_ms = INFINITY;
     int rc = SD_OK;
+    const size_t had[2] = {S->prep->Wh.size(), S->prep->Wsh.size()};
     auto trial = [&](const Plan& c) -> int {
         Search<T> t = *S;
         t.plan = c;
@@ -1200,6 +1201,17 @@ static int autotune(sd_ctx* ctx, Search<T>* S, cudaStream_t st) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    // the product tables that only a trial read (N^d elements each) go back; the others
+    // were there before, and graphs may hold them
+    const int keep_s_h = best.fft != SD_FFT_FULL ? S->G.s_h : 0;
+    for (int k = 0; k < 2; ++k) {
+        auto& cache = k ? S->prep->Wsh : S->prep->Wh;
+        for (size_t i = cache.size(); i-- > had[k];)
+            if (rc != SD_OK || cache[i].first != keep_s_h) {
+                pool_free(cache[i].second, st);
+                cache.erase(cache.begin() + (std::ptrdiff_t)i);
+            }
+    }
     if (rc != SD_OK) return rc;
     ctx->tuned[key] = best;
     S->plan = best;
