@@ -37,6 +37,18 @@ __host__ __device__ constexpr bool half_prefetch_w() { return LENF <= 256; }
 template <int LENF>
 __host__ __device__ constexpr bool half_prefetch_b() { return LENF != 256 && LENF != 384; }
 
+// Lines per CTA of the passes' form for few CTAs (2D jobs of few rotations), and whether it
+// pays against `ctas` CTAs of `lines` lines each.  Half a spectrum is half the lines, and
+// CTAs of 16 that leave SMs idle take as long as before or, with a transform more in the
+// chain, longer.  An FP64 CTA keeps its SM's pipe busy by itself, so the count of waves
+// decides, the smaller CTAs' at 1.15 (1.05 to 1.18 measured).
+constexpr int FEW_LINES = 4;
+inline bool few_pays(int64_t ctas, int lines) {
+    auto waves = [](int64_t n) { return (double)((n + 151) / 152); };
+    const int split = lines / FEW_LINES;
+    return 1.15 * waves(ctas * split) < split * waves(ctas);
+}
+
 template <typename T, int LENF, int TC>
 __host__ __device__ constexpr size_t cols_half_smem() {
     return ((size_t)TC * (col_pitch(LENF) + col_pitch(LENF / 2)) +
@@ -224,6 +236,92 @@ __global__ void __launch_bounds__(cta_threads_for<LENF>(TC), MB) k_cols_half(Col
     cols_half_body<T, LENF, TC, PRUNED, PACK>(a);
 }
 
+// The packing pass for launches of few CTAs (2D): FEW_LINES half columns per CTA, each
+// column and its mirror transformed by threads of their own at the same time, so the
+// chain is two transforms long where cols_half_body's is three.  us a launch by 16 (FP64
+// from 384 points 8) columns a CTA / this: FP64 N = 128 20 CTAs 74 / 29 (the full
+// spectrum's pass 45), 96 CTAs 74 / 61, 128 74 / 80, 192 (N = 96) 106 / 88; FP32, whose
+// SMs hold several CTAs, N = 192 30 CTAs 11.7 / 7.6, 72 11.8 / 9.8, 108 even, N = 128 72
+// CTAs 9.7 / 7.8, 128 9.6 / 10.1.
+template <typename T, int LENF>
+__host__ __device__ constexpr size_t cols_few_smem() {
+    return (size_t)2 * FEW_LINES * (col_pitch(LENF) + col_pitch(LENF / 2)) * sizeof(cplx<T>);
+}
+template <typename T, int LENF, bool PRUNED>
+__global__ void __launch_bounds__(cta_threads_for<LENF>(2 * FEW_LINES)) k_cols_few(ColArgs<T> a) {
+    using C = cplx<T>;
+    constexpr int LENI = LENF / 2, NH = LENI / 2, TC = FEW_LINES, NL = 2 * TC;
+    constexpr int NT = cta_threads_for<LENF>(NL);
+    static_assert(NT % NL == 0, "a thread keeps one line through the forward stages");
+    constexpr int LD = col_pitch(LENF), LDA = col_pitch(LENI);
+    constexpr int NB1 = LENF / plan_radix(LENF, 0);
+    constexpr int RL = plan_last_radix(LENF), PFL = LENF / RL;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* buf = reinterpret_cast<C*>(smem_raw);
+    C* acc = buf + NL * LD;
+    const int line = (int)threadIdx.x % NL;
+    const bool mirror = line >= TC;
+    const int kx = (int)blockIdx.x * TC + line % TC;
+    const bool ok = kx < NH;
+    const C* in = a.in + (int64_t)blockIdx.z * a.in_rot_stride + (mirror && kx ? LENI - kx : kx);
+    const C* W = a.W + kx + (mirror ? LENI * NH : 0);
+    C* out = a.out + (int64_t)blockIdx.z * a.out_rot_stride;
+    const int s = a.len_in;
+    const C zero = mk(T(0), T(0));
+    // as in cols_half_body: the input position, and the mode slot of an output
+    auto slot = [&](int i, int r) -> int {
+        if constexpr (PRUNED) {
+            return kept_out<LENF>(r) ? i + kept_slot<LENF>(r) : -1;
+        } else {
+            const int o = i + r * PFL;
+            return o < NH ? o : (o >= LENF - NH ? o - LENI : -1);
+        }
+    };
+    auto load = [&](int, int i, int r) -> C {
+        int e = i + r * NB1;
+        if constexpr (!PRUNED) {
+            e += a.s_h;
+            if (e >= LENF) e -= LENF;
+        }
+        const C v = (ok && e < s) ? in[e * LENI] : zero;
+        return mirror ? cconj(v) : v;
+    };
+    // the table's entries wait in the slots they are multiplied into
+    auto fetchW = [&] {
+#pragma unroll
+        for (int q = 0; q < (NL * PFL + NT - 1) / NT; ++q) {
+            const int t = threadIdx.x + q * NT;
+            if (t < NL * PFL)
+#pragma unroll
+                for (int r = 0; r < RL; ++r) {
+                    const int kp = slot(t / NL, r);
+                    if (kp < 0) continue;
+                    if (ok) copy_async(acc + line * LDA + kp, W + kp * NH);
+                    else acc[line * LDA + kp] = zero;
+                }
+        }
+        copy_commit();
+    };
+    auto emit = [&](int, int i, int r, C v) {
+        const int kp = slot(i, r);
+        if (kp >= 0 && ok) {
+            C* g = acc + line * LDA + kp;
+            *g = cmul(v, *g);
+        }
+    };
+    fftp_lines<C, LENF, false, NL, NT, LAY_COL, false, false, PRUNED>(buf, LD, a.twF, load, emit,
+                                                                      Hooks([&] { fetchW(); }, [&] { copy_wait(); }));
+    __syncthreads();
+    constexpr int NBI = LENI / plan_radix(LENI, 0);
+    auto sum = [&](int l, int i, int r) -> C {
+        const int p = i + r * NBI;
+        return cadd(acc[l * LDA + p], acc[(l + TC) * LDA + p]);
+    };
+    const int kxi = (int)blockIdx.x * TC + (int)threadIdx.x % TC;
+    PackEmit<C, LENI> emit_out{out, kxi, kxi < NH};
+    fftp_lines<C, LENI, true, TC, NT, LAY_COL, false, false, false>(buf, LDA, a.twI, sum, emit_out);
+}
+
 // Inverse y of half a spectrum (3D): columns (z, kx) of N points from the half
 // volume to packed lines.
 template <typename T, int LEN>
@@ -279,9 +377,9 @@ template <typename T, int LEN>
 __host__ __device__ constexpr bool rows_half_ahead() {
     return sizeof(T) == 4 && plan_radix(LEN, 1) != 0;
 }
-template <typename T, int LEN, int K>
+template <typename T, int LEN, int K, int TR>
 __host__ __device__ constexpr size_t rows_half_smem() {
-    constexpr int TR = lines_per_cta<T, LEN>(), NT = cta_threads<T, LEN>();
+    constexpr int NT = cta_threads_for<LEN>(TR);
     return (size_t)(TR * ((rows_half_ahead<T, LEN>() ? LEN : 0) + line_pitch(LEN)) + tw_count(LEN)) * sizeof(cplx<T>) +
            (K > 1 ? (size_t)NT * K * (sizeof(T) + sizeof(int)) : 0);
 }
@@ -295,11 +393,10 @@ __device__ __forceinline__ void copy_async16(void* dst, const void* src) {
 __device__ __forceinline__ float max_num(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double max_num(double a, double b) { return a > b || b != b ? a : b; }  // as fmax, but cheap
 
-template <typename T, int LEN, int K>
+template <typename T, int LEN, int K, int TR>
 __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
     using C = cplx<T>;
-    constexpr int TR = lines_per_cta<T, LEN>();
-    constexpr int NT = cta_threads<T, LEN>();
+    constexpr int NT = cta_threads_for<LEN>(TR);
     constexpr int LD = line_pitch(LEN);
     constexpr int NTW = tw_count(LEN);
     constexpr int NB1 = LEN / plan_radix(LEN, 0);
@@ -411,10 +508,10 @@ __device__ __forceinline__ void rows_half_body(const RowArgs<T>& a) {
     }
 }
 
-template <typename T, int LEN, int K>
-__global__ void __launch_bounds__(cta_threads<T, LEN>(), rows_half_min_ctas<T, LEN, K>())
+template <typename T, int LEN, int K, int TR>
+__global__ void __launch_bounds__(cta_threads_for<LEN>(TR), TR == FEW_LINES ? 0 : rows_half_min_ctas<T, LEN, K>())
 k_rows_half(RowArgs<T> a) {
-    rows_half_body<T, LEN, K>(a);
+    rows_half_body<T, LEN, K, TR>(a);
 }
 
 // The two halves of the table: W(kappa) / 2 and conj W(-kappa) / 2 times the phase of
@@ -464,11 +561,28 @@ static cudaError_t cols_half_launch(const ColArgs<T>& a, int batch, cudaStream_t
     return cudaGetLastError();
 }
 
+// 2D: N/2 columns a rotation.
+template <typename T, int LENF, int MB, bool PRUNED>
+static cudaError_t cols_half_2d(const ColArgs<T>& a, int batch, cudaStream_t st) {
+    constexpr int TC = lines_per_cta<T, LENF>();
+    const int64_t ctas = (int64_t)((a.ncols / 2 + TC - 1) / TC) * batch;
+    if (ctas > 0 && (sizeof(T) == 8 ? few_pays(ctas, TC) : ctas <= 96)) {
+        if (a.nouter != 1 || a.N != LENF / 2 || a.rot_fastest) return cudaErrorInvalidValue;
+        constexpr size_t smem = cols_few_smem<T, LENF>();
+        auto kern = k_cols_few<T, LENF, PRUNED>;
+        cudaError_t e = set_smem(kern, smem);
+        if (e != cudaSuccess) return e;
+        kern<<<dim3((a.ncols / 2 + FEW_LINES - 1) / FEW_LINES, 1, batch), cta_threads_for<LENF>(2 * FEW_LINES), smem, st>>>(a);
+        note_launch();
+        return cudaGetLastError();
+    }
+    return cols_half_launch<T, LENF, TC, MB, PRUNED, true>(a, batch, st);
+}
+
 template <typename T, int LENF>
 static cudaError_t cols_half_pruned(const ColArgs<T>& a, int batch, cudaStream_t st) {
     static_assert(prunable_len(LENF), "length not prunable");
-    if (a.ncols == a.N)  // 2D: N/2 columns in all, one width
-        return cols_half_launch<T, LENF, lines_per_cta<T, LENF>(), pruned_min_ctas<T, LENF, 2>(), true, true>(a, batch, st);
+    if (a.ncols == a.N) return cols_half_2d<T, LENF, pruned_min_ctas<T, LENF, 2>(), true>(a, batch, st);
     if constexpr (alt_cols_ok<T, LENF>()) {
         if (a.lines == LINES_NARROW)
             return cols_half_launch<T, LENF, alt_lines<T, LENF, 0>(), alt_min_ctas<T, LENF, 2, 0>(), true>(a, batch, st);
@@ -494,7 +608,7 @@ cudaError_t launch_cols_half_t(bool pruned, const ColArgs<T>& a, int batch, cuda
 #define SD_HALFF_CASE(L)                                                                                          \
     case L:                                                                                                       \
         return a.ncols == a.N                                                                                     \
-                   ? cols_half_launch<T, L, lines_per_cta<T, L>(), min_ctas_per_sm<T, L>(), false, true>(a, batch, st) \
+                   ? cols_half_2d<T, L, min_ctas_per_sm<T, L>(), false>(a, batch, st) \
                    : cols_half_launch<T, L, lines_per_cta<T, L>(), min_ctas_per_sm<T, L>(), false>(a, batch, st);
         SD_HALFF_CASE(16) SD_HALFF_CASE(32) SD_HALFF_CASE(48) SD_HALFF_CASE(64) SD_HALFF_CASE(96)
         SD_HALFF_CASE(128) SD_HALFF_CASE(192) SD_HALFF_CASE(256) SD_HALFF_CASE(384) SD_HALFF_CASE(512)
@@ -529,10 +643,9 @@ cudaError_t launch_pack_y_t(const ColArgs<T>& a, int batch, cudaStream_t st) {
     return cudaErrorInvalidValue;
 }
 
-template <typename T, int LEN, int K>
-static cudaError_t rows_half_launch(const RowArgs<T>& a, int batch, int* nparts, cudaStream_t st) {
-    constexpr int TR = lines_per_cta<T, LEN>();
-    constexpr int NT = cta_threads<T, LEN>();
+template <typename T, int LEN, int K, int TR>
+static cudaError_t rows_half_launch_tr(const RowArgs<T>& a, int batch, int* nparts, cudaStream_t st) {
+    constexpr int NT = cta_threads_for<LEN>(TR);
     if (a.nrows % 2 != 0 || a.N != LEN) return cudaErrorInvalidValue;
     const int ngroups = (a.nrows / 2 + TR - 1) / TR;
     if (nparts) *nparts = 0;
@@ -542,13 +655,29 @@ static cudaError_t rows_half_launch(const RowArgs<T>& a, int batch, int* nparts,
     G = G < 1 ? 1 : (G > half_row_most<K>() ? half_row_most<K>() : G);
     const int nb = (ngroups + G - 1) / G;
     if (nparts) *nparts = nb * K;
-    constexpr size_t smem = rows_half_smem<T, LEN, K>();
-    auto kern = k_rows_half<T, LEN, K>;
+    constexpr size_t smem = rows_half_smem<T, LEN, K, TR>();
+    auto kern = k_rows_half<T, LEN, K, TR>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(nb, batch), NT, smem, st>>>(a);
     note_launch();
     return cudaGetLastError();
+}
+
+// Fewer lines per CTA where few_pays (FP64, and FP32's short lists, whose insertions two
+// rows of a thread's outputs double): FP64 15 rotations at N = 128 22 -> 16 us, keeping four
+// 37 -> 26, 192 points 33 -> 20; FP32 keeping four 256 points, 320 CTAs 22 -> 16.  Long lists
+// pay for more partials to reduce: below half a wave only (72 CTAs at 96 points keeping 16
+// 74 -> 70, 192 CTAs 117 -> 143).
+template <typename T, int LEN, int K>
+static cudaError_t rows_half_launch(const RowArgs<T>& a, int batch, int* nparts, cudaStream_t st) {
+    constexpr int TR = lines_per_cta<T, LEN>();
+    if constexpr (sizeof(T) == 8 || K == 2 || K == 4) {
+        const int64_t ctas = (int64_t)((a.nrows / 2 + TR - 1) / TR) * batch;
+        if (few_pays(ctas, TR) && (K <= 4 || 2 * ctas <= 152))
+            return rows_half_launch_tr<T, LEN, K, FEW_LINES>(a, batch, nparts, st);
+    }
+    return rows_half_launch_tr<T, LEN, K, TR>(a, batch, nparts, st);
 }
 
 template <typename T>
