@@ -6,6 +6,10 @@
 
 namespace sd {
 
+// SMs of a GB300.  Rules that cut work for a wave of CTAs count with it: they are lines
+// measured on that chip, not properties of whatever device is present.
+constexpr int GPU_SMS = 152;
+
 // Counts kernel launches made by the library (defined in api.cu).
 void note_launch(int n = 1);
 

@@ -505,7 +505,7 @@ template <typename T>
 cudaError_t launch_gather(const GatherArgs<T>& args, int dim, cudaStream_t st) {
     if (args.P == 0 || args.m2 == 0) return cudaSuccess;
     GatherArgs<T> a = args;
-    constexpr int64_t CTAS = 4 * 152;  // one wave
+    constexpr int64_t CTAS = 4 * GPU_SMS;  // one wave
     bool apart = false;
     // Samples per CTA: at most what its stage holds, at least one per warp, the wave's CTAs
     // shared out evenly among the poses (512 poses x 50 samples in chunks of 48 took a second
@@ -522,7 +522,7 @@ cudaError_t launch_gather(const GatherArgs<T>& args, int dim, cudaStream_t st) {
         const int64_t want = ((a.m2 + per_pose - 1) / per_pose + 7) / 8 * 8;
         a.chunk = (int)(want < 8 ? 8 : (want > most ? most : want));
         const unsigned ctas = (unsigned)((a.m2 + a.chunk - 1) / a.chunk);
-        a.few = a.chunk <= GA_THREADS / 4 && (sizeof(T) == 4 || dim == 3 || ctas * a.P <= 152);
+        a.few = a.chunk <= GA_THREADS / 4 && (sizeof(T) == 4 || dim == 3 || ctas * a.P <= GPU_SMS);
         apart = ctas * a.P > (sizeof(T) == 4 ? 2 : 1) * CTAS;
         return dim3(ctas, (unsigned)a.P);
     };

@@ -23,7 +23,7 @@ namespace sd {
 
 // Twiddles in shared memory where that costs no resident CTA: a 384-point CTA (line
 // buffer 49 KB, mode buffer 25 KB) would miss its third, and 512 points (99 KB)
-// measured faster through L1 (12 rotations at N = 256: 1171 against 1273 us; 256 points
+// measured faster through L1 (12 rotations at N = 256: 894 against 1038 us; 256 points
 // the other way, 68 rotations at N = 128: 562 against 524).
 template <int LENF>
 __host__ __device__ constexpr bool half_tw_smem() { return LENF <= 256; }
@@ -44,7 +44,7 @@ __host__ __device__ constexpr bool half_prefetch_b() { return LENF != 256 && LEN
 // decides, the smaller CTAs' at 1.15 (1.05 to 1.18 measured).
 constexpr int FEW_LINES = 4;
 inline bool few_pays(int64_t ctas, int lines) {
-    auto waves = [](int64_t n) { return (double)((n + 151) / 152); };
+    auto waves = [](int64_t n) { return (double)((n + GPU_SMS - 1) / GPU_SMS); };
     const int split = lines / FEW_LINES;
     return 1.15 * waves(ctas * split) < split * waves(ctas);
 }
@@ -651,7 +651,7 @@ static cudaError_t rows_half_launch_tr(const RowArgs<T>& a, int batch, int* npar
     if (nparts) *nparts = 0;
     if (ngroups == 0 || batch == 0) return cudaSuccess;
     const int64_t total = (int64_t)ngroups * batch;
-    int G = (int)(total / (half_row_wave<K>() * 152));
+    int G = (int)(total / (half_row_wave<K>() * GPU_SMS));
     G = G < 1 ? 1 : (G > half_row_most<K>() ? half_row_most<K>() : G);
     const int nb = (ngroups + G - 1) / G;
     if (nparts) *nparts = nb * K;
@@ -674,7 +674,7 @@ static cudaError_t rows_half_launch(const RowArgs<T>& a, int batch, int* nparts,
     constexpr int TR = lines_per_cta<T, LEN>();
     if constexpr (sizeof(T) == 8 || K == 2 || K == 4) {
         const int64_t ctas = (int64_t)((a.nrows / 2 + TR - 1) / TR) * batch;
-        if (few_pays(ctas, TR) && (K <= 4 || 2 * ctas <= 152))
+        if (few_pays(ctas, TR) && (K <= 4 || 2 * ctas <= GPU_SMS))
             return rows_half_launch_tr<T, LEN, K, FEW_LINES>(a, batch, nparts, st);
     }
     return rows_half_launch_tr<T, LEN, K, TR>(a, batch, nparts, st);

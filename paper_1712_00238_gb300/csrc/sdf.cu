@@ -330,7 +330,7 @@ __device__ __forceinline__ bool node_far(const T* nd, const float lo[3], const f
 // cylinder (50,342, 20,000) 0.17 ms.
 constexpr int TREE_NW = 8;
 // Two queries a lane where that still gives every SM two CTAs.
-constexpr int64_t TREE_PAIR_MIN = 64 * 2 * 152;
+constexpr int64_t TREE_PAIR_MIN = 64 * 2 * GPU_SMS;
 
 template <typename T, int Q>
 __global__ void __launch_bounds__(32 * TREE_NW, sizeof(T) == 4 ? 4 : 0) k_sdf_tree(SdfArgs<T> a, const T* nodes, const float* tile_box,
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(32 * TREE_NW, sizeof(T) == 4 ? 4 : 0) k_sdf_tr
 // Membership of the listed queries from the sum over every sample.  Work items
 // (256 queries, a share of the tiles) are dealt to a fixed grid, so that a few
 // queries against many samples still fill it; a warp adds a query's shares.
-constexpr int LIST_CTAS = 152 * 8;
+constexpr int LIST_CTAS = GPU_SMS * 8;
 __host__ __device__ __forceinline__ int list_splits(int chunks, int64_t n_tiles) {
     const int s = LIST_CTAS / (chunks > 0 ? chunks : 1);
     return s < 1 ? 1 : (s > n_tiles ? (int)n_tiles : s);
@@ -955,7 +955,7 @@ static int sdf_splits(int64_t query_blocks, int64_t tiles, int most = 64) {
 // about 20,000 samples 1,107 / 290 (in a cube; 525 / 290 in a band at the boundary),
 // 2,000 about 300,000 14,190 / 1,880 (3,600 / 1,230); FP64, 500 about 5,000 3,420 / 1,140.
 static int sum_splits(int64_t groups, int64_t tiles) {
-    const int64_t s = std::min((16 * 152 + groups - 1) / groups, std::min<int64_t>(tiles / 4, 256));
+    const int64_t s = std::min((16 * GPU_SMS + groups - 1) / groups, std::min<int64_t>(tiles / 4, 256));
     return s < 1 ? 1 : (int)s;
 }
 
@@ -1027,7 +1027,7 @@ static cudaError_t launch_nearest(const SdfArgs<T>& a, int dim, cudaStream_t st)
         note_launch();
         if (!a.pmc_override) {
             k_sdf_wind_list<T><<<LIST_CTAS, SDF_TILE, 0, st>>>(a, list, list_n, part);
-            k_sdf_wind_list_finish<T><<<152, SDF_TILE, 0, st>>>(a, list, list_n, part);
+            k_sdf_wind_list_finish<T><<<GPU_SMS, SDF_TILE, 0, st>>>(a, list, list_n, part);
             note_launch(2);
         }
     }
