@@ -744,8 +744,8 @@ __global__ void __launch_bounds__(SDF_TILE) k_sdf_sum(SdfArgs<T> a, int tiles_pe
 // The same sum (3D, Eq. 15 with a truncation) over the tree: one CTA per 32
 // queries as in k_sdf_tree, tiles tested 32 at a time against the warp's reach
 // (1 + eps) max|xi|, each warp taking one of a tile's sub-tiles unless it lies beyond
-// every lane's own reach: what is skipped holds no pair that passes Eq. 17t.  What a lane adds, and in which order, does not depend on what
-// is skipped.  (One CTA per 256 queries, in lock-step over whole tiles: 14.0 ms for
+// every lane's own reach: what is skipped holds no pair that passes Eq. 17t.  What a lane
+// adds, and in which order, does not depend on what is skipped.  (One CTA per 256 queries, in lock-step over whole tiles: 14.0 ms for
 // 5,000 spheres.)  Queries too few to fill the GPU have the tiles dealt to several CTAs
 // (grid y, sum_splits; in turn, as a group's near tiles are neighbours), a partial sum
 // each with its compensation, which k_sdf_sum_finish adds.
